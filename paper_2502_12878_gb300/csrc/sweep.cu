@@ -470,6 +470,93 @@ __global__ void apply_rowmajor(const double* w, const int32_t* idx, int64_t nc, 
     }
 }
 
+// Tiles: the caller's stencils are row-major, so a thread that walks its own
+// row reads one 8-byte word of a sector at a time, n words from its
+// neighbour's.  Here each warp copies 32 whole rows - one contiguous run - into
+// shared memory with 16-byte asynchronous copies (whole lines; no registers
+// held in flight), and thread = row reads its row back, E entries at a time (the pairs
+// of an even n leave at most 4-way bank conflicts, at n a multiple of 8; an odd
+// row pitch leaves none), for the same fma chain in support order.
+// Bound by HBM and the FP64 pipe together (376 MB and n FP64 instructions a
+// row at 1M rows, n = 30: 55 and 50 us) through the copies' latency: one tile a
+// warp, and as many warps as shared memory holds, each its own block (blocks
+// pack it better).  1M rows: n = 12 47 -> 32 us, n = 30 180 -> 75, n = 56
+// 356 -> 144.  Two tiles a warp on half the warps: 90 us at n = 30; four
+// warps a block: 92; copies into an odd pitch, which need 4- and 8-byte
+// instructions: 101; bulk copies (TMA) on an mbarrier: 79.
+static constexpr int APPLY_WARPS = 1;
+
+template <int E>
+__global__ void __launch_bounds__(32 * APPLY_WARPS)
+apply_tiles(const double* __restrict__ w, const int32_t* __restrict__ idx, int64_t nc, int n,
+            const double* __restrict__ u, double* __restrict__ Lu) {
+    extern __shared__ __align__(16) unsigned char apply_smem[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int ent = SLICE * n;
+    unsigned char* ws = apply_smem + (size_t)wib * ent * 12;
+    unsigned char* is = ws + (size_t)ent * 8;
+    const uint32_t wd = (uint32_t)__cvta_generic_to_shared(ws);
+    const uint32_t id = (uint32_t)__cvta_generic_to_shared(is);
+    const double* wr = reinterpret_cast<const double*>(ws) + lane * n;
+    const int32_t* ir = reinterpret_cast<const int32_t*>(is) + lane * n;
+    const int64_t nfull = nc / SLICE;
+    const int64_t stride = (int64_t)gridDim.x * APPLY_WARPS;
+    const int64_t t0 = (int64_t)blockIdx.x * APPLY_WARPS + wib;
+    for (int64_t t = t0; t < nfull; t += stride) {
+        const char* wg = reinterpret_cast<const char*>(w + t * ent);
+        const char* ig = reinterpret_cast<const char*>(idx + t * ent);
+        for (int o = lane * 16; o < ent * 4; o += 512)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(id + o), "l"(ig + o)
+                         : "memory");
+        for (int o = lane * 16; o < ent * 8; o += 512)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(wd + o), "l"(wg + o)
+                         : "memory");
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        double acc = 0.0;
+        int j = 0;
+        for (; j + 8 <= n; j += 8) {
+            int32_t c[8];
+            double uv[8], wv[8];
+#pragma unroll
+            for (int k = 0; k < 8; k += E) {
+                if constexpr (E == 2) {
+                    const int2 x = *reinterpret_cast<const int2*>(ir + j + k);
+                    c[k] = x.x;
+                    c[k + 1] = x.y;
+                } else {
+                    c[k] = ir[j + k];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) uv[k] = __ldg(u + c[k]);
+#pragma unroll
+            for (int k = 0; k < 8; k += E) {
+                if constexpr (E == 2) {
+                    const double2 x = *reinterpret_cast<const double2*>(wr + j + k);
+                    wv[k] = x.x;
+                    wv[k + 1] = x.y;
+                } else {
+                    wv[k] = wr[j + k];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc = __fma_rn(wv[k], uv[k], acc);
+        }
+        for (; j < n; ++j) acc = __fma_rn(wr[j], __ldg(u + ir[j]), acc);
+        Lu[t * SLICE + lane] = acc;
+        __syncwarp();   // the tile is read before the next copies overwrite it
+    }
+    // the rows of a last partial tile, straight from global memory
+    const int64_t r = nfull * SLICE + lane;
+    if (t0 == nfull % stride && r < nc) {
+        double acc = 0.0;
+        for (int j = 0; j < n; ++j)
+            acc = __fma_rn(w[r * n + j], __ldg(u + idx[r * n + j]), acc);
+        Lu[r] = acc;
+    }
+}
+
 // ------------------------------------------------------------ host side
 // One graph-mode step launch.  With programmatic stream serialization (pdl)
 // the next launch of a captured chunk can start while this one drains.  The
@@ -1266,6 +1353,24 @@ extern "C" int rbffd_apply(const double* w, const int32_t* idx, int64_t nc, int 
     if (nc == 0) return RBFFD_OK;
     RBFFD_ARG(w && idx && u && Lu, "rbffd_apply: NULL argument");
     int sms = device_sm_count();
+    // whole-row tiles where the 16-byte copies may start at every tile and a
+    // tile fits a block's shared memory (n <= 586); else a thread per row
+    const size_t smem = (size_t)APPLY_WARPS * SLICE * n * 12;
+    if (smem <= 220 * 1024 &&
+        (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(idx)) % 16 == 0) {
+        const void* fn = n % 2 ? (const void*)apply_tiles<1> : (const void*)apply_tiles<2>;
+        if (smem > 48 * 1024)
+            RBFFD_CHECK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem));
+        const int64_t ntiles = (nc + SLICE - 1) / SLICE;
+        const int64_t per_sm = std::min<int64_t>(32, (227 * 1024) / (int64_t)(smem + 1024));
+        const int64_t grid =
+            std::min<int64_t>((ntiles + APPLY_WARPS - 1) / APPLY_WARPS, (int64_t)sms * per_sm);
+        void* args[] = {(void*)&w, (void*)&idx, (void*)&nc, (void*)&n, (void*)&u, (void*)&Lu};
+        RBFFD_CHECK_CUDA(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(32 * APPLY_WARPS), args,
+                                          smem, as_stream(stream)));
+        return RBFFD_OK;
+    }
     int64_t blocks = std::min<int64_t>((nc + 255) / 256, (int64_t)sms * 16);
     apply_rowmajor<<<(unsigned)blocks, 256, 0, as_stream(stream)>>>(w, idx, nc, n, u, Lu);
     RBFFD_CHECK_CUDA(cudaGetLastError());
