@@ -76,7 +76,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
 }
 
 // the iterate at slot c: from the block's halo window [lo, lo + W) in shared
-// memory, else through L2 (.cg: other blocks rewrite the iterate between steps)
+// memory, else a load through L1 (other blocks rewrite the iterate between steps,
+// each step behind an acquire)
 template <class T>
 __device__ __forceinline__ T res_u(const T* hs, int32_t lo, uint32_t W, const T* __restrict__ u,
                                    int32_t c) {
