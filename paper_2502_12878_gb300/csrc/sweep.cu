@@ -458,6 +458,124 @@ __global__ void sum_to_norm(const double* part, int nparts, double* norm_out) {
     if (threadIdx.x == 0) *norm_out = sqrt(sh[0]);
 }
 
+// All iterations in one cooperative launch: y_{k+1} = 2^-e_k W_II y_k, where e_k
+// is the exponent of max |y_k| (boundary slots 0 in both buffers).  Scaling by a
+// power of two is exact, so no iteration rounds its vector to unit norm, and
+// what a step needs of the previous one - a maximum - does not depend on the
+// order of the blocks; only the last two iterations sum squares, for
+// rho = ||W y|| / ||y||.  One counter barrier an iteration, as in the
+// persistent sweeps; res[k % 3] holds max |y_k| (IEEE bits).
+// What bounds it: the sweep's own limits at 1M rows (HBM and the FP64 pipe), the
+// barrier and one dependent L2 round trip on small plans.  Before, three
+// launches an iteration (a sweep, a sum, a
+// scaling); 200 iterations: 10k rows, n = 12 2.94 -> 0.79 ms; 90k, n = 30 4.18
+// -> 2.02; 1M, n = 12 10.6 -> 6.9, n = 30 17.4 -> 14.0; 3D 205k, n = 70 9.1 -> 9.0
+// (10.6 with gathers that skip L1).
+template <int NN>
+__global__ void __launch_bounds__(STEP_THREADS, NN > 0 ? 4 : 1)
+power_persist(StepArgs A, StepCtrl* c, long long iters, double* part) {
+    __shared__ double ws[STEP_THREADS / 32];
+    __shared__ double s_sc;
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = step_warp(A);
+    const int64_t nw = (int64_t)gridDim.x * (STEP_THREADS / 32);
+    const long long lim = ((volatile StepCtrl*)c)->spin_limit;
+    const long long spin = lim > 0 ? lim : (long long)SPIN_LIMIT_CYCLES;
+    for (long long k = 0; k < iters; ++k) {
+        const double* v = (k & 1) ? A.u1 : A.u0;
+        double* y = (k & 1) ? A.u0 : A.u1;
+        if (threadIdx.x == 0) {
+            const unsigned ex = (unsigned)(ld_relaxed(&c->res[k % 3]) >> 52);
+            s_sc = bitsd(ex >= 1u && ex <= 2045u ? (unsigned long long)(2046u - ex) << 52
+                                                 : 0x3ff0000000000000ull);
+        }
+        __syncthreads();
+        const double sc = s_sc;
+        const bool last2 = k + 2 >= iters;
+        double s = 0.0;
+        unsigned long long m = 0;
+        for (int64_t sl = warp; sl < A.nslices; sl += nw) {
+            const int64_t row = sl * SLICE + lane;
+            const int64_t base = sl * (int64_t)A.n * SLICE + lane;
+            const int4 sb = A.col16 ? __ldg(A.sbase + sl) : make_int4(-1, -1, -1, -1);
+            if (NN > 0 && NN <= PF64_MAX_N && lane == 0)
+                prefetch_planes<MODE_SWEEP64>(A, sl + nw);
+            if (row < A.NI) {
+                const double acc =
+                    sb.x >= 0 ? row_dot<NN, true, true, double>(A.w64 + base, A.col16 + base, sb,
+                                                                v, A.n)
+                              : row_dot64<NN, true>(A.w64 + base, A.col + base, v, A.n);
+                const double yv = __dmul_rn(acc, sc);
+                y[row] = yv;
+                m = max(m, abs_bits(yv));
+                if (last2) s = __fma_rn(yv, yv, s);
+            }
+        }
+        if (last2) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) ws[threadIdx.x >> 5] = s;
+        }
+        m = block_max_bits(m);   // a block barrier: ws is complete behind it
+        int ok = 1;
+        if (threadIdx.x == 0) {
+            if (last2) {
+                double t = 0.0;
+                for (int w = 0; w < STEP_THREADS / 32; ++w) t += ws[w];
+                part[(k + 1 == iters ? gridDim.x : 0) + blockIdx.x] = t;
+                if (k + 1 == iters && blockIdx.x == 0) part[2 * gridDim.x] = sc;
+            }
+            if (blockIdx.x == 0) st_relaxed(&c->res[(k + 2) % 3], 0ull);
+            red_max_relaxed(&c->res[(k + 1) % 3], m);
+            red_add_release(&c->arrivals, 1ull);
+            const unsigned long long target = (unsigned long long)(k + 1) * gridDim.x;
+            const long long t0 = clock64();
+            while (ld_acquire(&c->arrivals) < target)
+                if (clock64() - t0 > spin) {
+                    atomicExch(&c->done, DONE_TIMEOUT);
+                    ok = 0;
+                    break;
+                }
+        }
+        if (!__syncthreads_and(ok)) return;
+    }
+}
+
+// max |v| over the interior slots into *out (IEEE bits)
+__global__ void vec_max(const double* __restrict__ v, int64_t NI, unsigned long long* out) {
+    unsigned long long m = 0;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
+         p += (int64_t)gridDim.x * blockDim.x)
+        m = max(m, abs_bits(v[p]));
+    m = block_max_bits(m);
+    if (threadIdx.x == 0) red_max_relaxed(out, m);
+}
+
+// rho = sqrt(sum s1) / (sc sqrt(sum s0)), the sums in a fixed order; s0 is null
+// for a single iteration (then the start vector's squares sv, sc unscaled).
+// NaN where sv's sum is 0 or not finite: such a start vector has no direction.
+__global__ void power_rho(const double* sv, int nv, const double* s0, int n0, const double* s1,
+                          int n1, const double* sc, double* rho) {
+    __shared__ double sh[3][256];
+    double a = 0.0, b = 0.0, v = 0.0;
+    for (int i = threadIdx.x; i < n0; i += blockDim.x) a += s0[i];
+    for (int i = threadIdx.x; i < n1; i += blockDim.x) b += s1[i];
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) v += sv[i];
+    sh[0][threadIdx.x] = a;
+    sh[1][threadIdx.x] = b;
+    sh[2][threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o)
+            for (int q = 0; q < 3; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double vv = sh[2][0], yy = s0 ? sh[0][0] : vv;
+        *rho = vv > 0.0 && isfinite(vv) ? sqrt(sh[1][0]) / (sqrt(yy) * *sc) : __longlong_as_double(0x7ff8000000000000ll);
+    }
+}
+
 // ------------------------------------------------------------ apply (Eq. 1)
 __global__ void apply_rowmajor(const double* w, const int32_t* idx, int64_t nc, int n,
                                const double* u, double* Lu) {
@@ -1887,11 +2005,9 @@ extern "C" int rbffd_solve_explicit(rbffd_plan* p, const double* f, double* u, d
     return done_status(done);
 }
 
-extern "C" int rbffd_stable_dt(rbffd_plan* p, const double* v0, int iters, double safety,
-                               double* h_dt_out, double* h_rho_out, void* stream) {
-    clear_error();
-    RBFFD_ARG(p && v0 && iters >= 1 && safety > 0.0, "rbffd_stable_dt: bad argument");
-    cudaStream_t s = as_stream(stream);
+// the power iteration as three launches an iteration
+static int power_stepwise(rbffd_plan* p, const StepArgs& A, const double* v0, int iters,
+                          double* rho, cudaStream_t s) {
     const int sms = device_sm_count();
     // v lives in u[0] (slot order; boundary slots 0), y in scratch[1024 ..]
     double* v = p->u[0];
@@ -1905,7 +2021,6 @@ extern "C" int rbffd_stable_dt(rbffd_plan* p, const double* v0, int iters, doubl
     sum_to_norm<<<1, 256, 0, s>>>(part, nparts, nrm);
     power_scale<<<sms * 8, 256, 0, s>>>(nrm, y, v, p->NI);
     RBFFD_CHECK_CUDA(cudaGetLastError());
-    StepArgs A = make_args(p);
     typedef void (*PowFn)(StepArgs, const double*, double*, double*);
     PowFn pf;
     switch (p->n) {
@@ -1928,9 +2043,78 @@ extern "C" int rbffd_stable_dt(rbffd_plan* p, const double* v0, int iters, doubl
         power_scale<<<sms * 8, 256, 0, s>>>(nrm, y, v, p->NI);
     }
     RBFFD_CHECK_CUDA(cudaGetLastError());
-    double rho = 0.0;
-    RBFFD_CHECK_CUDA(cudaMemcpyAsync(&rho, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(rho, nrm, sizeof(double), cudaMemcpyDeviceToHost, s));
     RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
+    return RBFFD_OK;
+}
+
+// the power iteration in one cooperative launch; *done false where the device
+// cannot hold the grid at once
+static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int iters,
+                        double* rho, bool* done, cudaStream_t s) {
+    const int sms = device_sm_count();
+    typedef void (*PowFn)(StepArgs, StepCtrl*, long long, double*);
+    PowFn pf;
+    switch (p->n) {
+        case 12: pf = power_persist<12>; break;
+        case 30: pf = power_persist<30>; break;
+        case 56: pf = power_persist<56>; break;
+        case 70: pf = power_persist<70>; break;
+        default: pf = power_persist<0>; break;
+    }
+    const int grid = persistent_grid((StepFn)(void*)pf, p);
+    const int nparts = 1024;
+    if (2 * grid + 1 > 2 * nparts) return RBFFD_OK;   // scratch holds 4096 partial sums
+    double* part = p->scratch + 8;
+    int st = ctrl_reset(p, 0.0, 0.0, iters, s);
+    if (st) return st;
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[0], 0, sizeof(double) * p->N, s));
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[1], 0, sizeof(double) * p->N, s));
+    gather_f<<<sms * 8, 256, 0, s>>>(v0, p->row_of_slot, p->NI, p->u[0]);
+    vec_max<<<sms, 256, 0, s>>>(p->u[0], p->NI, &p->ctrl->res[0]);
+    norm_partials<<<nparts, 256, 0, s>>>(p->u[0], p->NI, part + 2 * nparts);
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    StepCtrl* c = p->ctrl;
+    long long n_it = iters;
+    StepArgs a = A;
+    void* args[] = {(void*)&a, (void*)&c, (void*)&n_it, (void*)&part};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)pf, dim3(grid),
+                                                      dim3(STEP_THREADS), args, 0, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return RBFFD_OK;
+    }
+    RBFFD_CHECK_CUDA(e);
+    const bool one = iters == 1;   // else the last iteration but one summed its squares
+    power_rho<<<1, 256, 0, s>>>(part + 2 * nparts, nparts, one ? nullptr : part, one ? 0 : grid,
+                                part + grid, grid, part + 2 * grid, p->scratch);
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    int stopped = 0;
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(&stopped, &p->ctrl->done, sizeof(int),
+                                     cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(rho, p->scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
+    if (stopped == DONE_TIMEOUT) return done_status(DONE_TIMEOUT);
+    *done = true;
+    return RBFFD_OK;
+}
+
+extern "C" int rbffd_stable_dt(rbffd_plan* p, const double* v0, int iters, double safety,
+                               double* h_dt_out, double* h_rho_out, void* stream) {
+    clear_error();
+    RBFFD_ARG(p && v0 && iters >= 1 && safety > 0.0, "rbffd_stable_dt: bad argument");
+    cudaStream_t s = as_stream(stream);
+    StepArgs A = make_args(p);
+    double rho = 0.0;
+    bool done = false;
+    if (p->NN == 0) {   // (the Neumann update between iterations needs launches of its own)
+        int st = power_launch(p, A, v0, iters, &rho, &done, s);
+        if (st) return st;
+    }
+    if (!done) {
+        int st = power_stepwise(p, A, v0, iters, &rho, s);
+        if (st) return st;
+    }
     if (!(rho > 0.0) || !isfinite(rho)) {
         set_error("rbffd_stable_dt: spectral radius estimate is %g", rho);
         return RBFFD_ERR_NONFINITE;

@@ -1,0 +1,48 @@
+"""The power iteration's single launch (plans without Neumann nodes) against the oracle's
+iteration: one, two and many iterations (the norms come from different kernels), stencil sizes
+with and without a compiled kernel, node orders, int32 indices, one partial slice; vectors with
+no direction or with NaN are refused."""
+import numpy as np
+import pytest
+
+import rbffd_inputs as gen
+from oracle_problem import build
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2502_12878_gb300 import build as nvbuild
+    nvbuild.build()
+    import paper_2502_12878_gb300 as m
+    m.lib()
+    return m
+
+
+def T(x):
+    return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+@pytest.mark.parametrize("d,Kg,m,n,flags", [(2, 60, 2, 12, 0), (2, 45, 4, 30, 64),
+                                            (2, 45, 4, 31, 2), (2, 30, 4, 30, 32),
+                                            (2, 40, 6, 56, 0), (3, 12, 4, 70, 0),
+                                            (2, 4, 1, 6, 0)])
+def test_radius_equals_the_oracles(rb, orc, d, Kg, m, n, flags):
+    p = build(orc, d, Kg, m, seed=17, n=n)
+    plan = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w), flags, 3)
+    v0 = gen.random_vector(p.NI, 5)
+    # each iteration's sums of n + N terms round within (n + N) 2^-53 of the exact ones and
+    # the radius is stationary to first order; the repository's bound is 1e-9
+    for iters in (1, 2, 3, 200):
+        rho = orc.power_rho(p.w, p.idx, p.interior, p.N, v0, iters)
+        for scale in (1.0, 1e-100, 1e100):
+            got = plan.stable_dt(T(v0 * scale), iters, 1.05)[1]
+            assert abs(got - rho) <= 1e-9 * rho
+    # no direction: zero, NaN, squares that underflow or overflow
+    for bad in (np.zeros(p.NI), np.full(p.NI, np.nan), v0 * 1e-200, v0 * 1e200):
+        with pytest.raises(rb.RbffdError):
+            plan.stable_dt(T(bad), 5)
