@@ -323,7 +323,11 @@ RBFFD_API int rbffd_fp64_fma_rate(int64_t iters, double* h_fma_per_s, double* h_
  * the iterate; it fits while the plan's share per SM does (about 102,000
  * interior rows at n = 30 in FP64 with 16-bit codes, 175,000 for the FP32
  * inner sweep); a _RESIDENT plan that does not fit returns
- * RBFFD_ERR_CAPACITY from its first solve.  A Morton plan created with a
+ * RBFFD_ERR_CAPACITY from its first solve.  Unless a reach is fixed by
+ * rbffd_plan_set_resident_halo, _RESIDENT and _AUTO plans that fit run it linked:
+ * blocks pass each other the rows that they read, tagged with their step, so that
+ * a step waits for its neighbours' rows instead of a barrier of all blocks (16 x 8
+ * bytes a row of device memory more).  A Morton plan created with a
  * flag that allows the resident or split launch, whose share per SM is at
  * least two slices and fits one of them, orders each share's rows with the
  * rows whose supports lie inside the share first, each group in Morton
@@ -356,12 +360,13 @@ RBFFD_API int rbffd_plan_set_neumann(rbffd_plan* plan, int64_t NN, const int32_t
                                      const double* g, void* stream);
 /*
  * rbffd_plan_set_wait - the in-kernel waits of the persistent launch (the
- * end-of-step grid barrier): each gives up after timeout_ms (<= 0: the
+ * end-of-step grid barrier; linked: the waits for other blocks' rows and stop
+ * decisions): each gives up after timeout_ms (<= 0: the
  * default, about 2 s; at most 60,000), measured in SM clock cycles at the
  * device's maximum clock, and the solve then returns RBFFD_ERR_TIMEOUT.
  * held_arrivals (0..1024, normally 0) is a failure injection for testing that
- * path: the barrier waits for that many arrivals beyond the grid's, which
- * never come, so every block gives up after the timeout and returns.  Takes
+ * path: the barrier waits for that many arrivals beyond the grid's (linked: the
+ * stop decisions are withheld), which never come, so every block gives up after the timeout and returns.  Takes
  * effect from the next solve; graph-mode steps have no waits.
  */
 RBFFD_API int rbffd_plan_set_wait(rbffd_plan* plan, double timeout_ms, int held_arrivals);
@@ -418,7 +423,8 @@ RBFFD_API int rbffd_solve_explicit(rbffd_plan* plan, const double* f, double* u,
  * launched; h_shape[4], the autotuned launch shape (register budget, blocks
  * per SM; 0 blocks per SM = the persistent launch, -1 = the resident launch,
  * whose first entry is then its block size in units of 512 threads, + 4
- * when it stages far lists (every gather from shared memory), -2 = the split
+ * when it stages far lists (every gather from shared memory), + 8 when it
+ * runs linked (without a grid barrier), -2 = the split
  * launch, whose first entry is its block size in units of 512 threads;
  * blocks per SM + 16 = graph-replayed steps launched as programmatic
  * dependent launches) of the FP64 sweep and of the FP32 inner sweep.

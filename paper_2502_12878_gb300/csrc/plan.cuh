@@ -100,6 +100,19 @@ struct rbffd_plan {
     uint16_t* fl_idx[2] = {nullptr, nullptr};
     int32_t* fl_off[2] = {nullptr, nullptr};
     int32_t* fl_slot[2] = {nullptr, nullptr};
+    // linked launch (step_link.cuh), built when the tuner first considers it: local
+    // indices, halo lists, the entry ring and its residual and decision words, and
+    // the tags used so far
+    bool link[2] = {false, false};      // the step loop of each mode runs as it
+    bool lk_built = false, lk_ok = false;
+    int lk_grid = 0;
+    int64_t lk_max = 0;
+    uint16_t* lk_idx = nullptr;
+    int32_t* lk_off = nullptr;
+    int32_t* lk_slot = nullptr;
+    unsigned long long* lk_x = nullptr;   // ring, residuals and decisions, one allocation
+    size_t lk_bytes = 0;
+    unsigned long long lk_epoch = 0;
     int64_t res_halo[2] = {0, 0};       // and its halo reach (slots beyond a block's rows)
     int64_t res_halo_set = -2;          // a reach fixed by rbffd_plan_set_resident_halo (-2: tuned)
     int res_threads_set = 0;            // block size fixed by rbffd_plan_set_block (0: tuned)

@@ -191,7 +191,26 @@ struct StepArgs {
     // split launch: per block (SM) the number of leading slices of its share
     // that are inner rows only (plans ordered inner rows first)
     const int32_t* inner;
+    // linked launch (step_link.cuh): every entry's local index (own row of the
+    // block, or its rows' count plus a place in the halo list), per block the
+    // sorted slots of other blocks and of the boundary that its rows read, the
+    // largest such list, the entry ring, residual and decision words, and the
+    // tag before this run's first
+    const uint16_t* lk_idx;   // [nslices][n][32]
+    const int32_t* lk_off;    // [blocks + 1]
+    const int32_t* lk_slot;
+    int64_t lk_max;
+    unsigned long long* lk_x;     // [LINK_RING][NI] entries of one (FP32) or two words
+    unsigned long long* lk_res;   // [LINK_RING][blocks] two-word entries
+    unsigned long long* lk_dec;   // [LINK_RING]
+    unsigned lk_epoch;
 };
+
+// iterates in the linked launch's ring, and how many steps a block may be ahead
+// of the slowest (its stop decision): an entry is overwritten LINK_RING steps later, when
+// every block has finished the steps up to LINK_LAG back, so LINK_RING >= LINK_LAG + 2
+static constexpr int LINK_RING = 8;
+static constexpr int LINK_LAG = 5;
 
 // The warp's first slice.  Large plans give each block runs of consecutive
 // slices (their gathers share the SM's L1); plans with fewer slices than the
@@ -580,6 +599,10 @@ StepFn pick_resident_wide(int mode, int n, bool i16);
 // the resident launch with far lists (step_res_far.cu), `threads` a block
 // (nullptr where that block size is not compiled for n)
 StepFn pick_resident_far(int mode, int n, int threads);
+// the linked launch (step_link.cu; nullptr where `threads` is not compiled for
+// n) and its dynamic shared memory for halo lists of at most `halo` slots
+StepFn pick_link(int mode, int n, int threads);
+unsigned link_smem(int64_t nslices, int n, int mode, int grid, int64_t halo);
 // dynamic shared memory of a resident launch of `grid` blocks whose halo
 // window reaches `halo` slots beyond each block's rows on either side, with
 // room for `extra` more values behind it (the far values)

@@ -25,7 +25,8 @@
 //              barrier whose waits are bounded in time (RBFFD_ERR_TIMEOUT);
 //              the stop rule for a step is applied after the next one.
 //  resident    the persistent launch with each block's stencil planes held
-//              in shared memory (step_res.cuh).
+//              in shared memory (step_res.cuh), or the linked launch, which
+//              exchanges rows between blocks without a barrier (step_link.cuh).
 // The residual max-norm is reduced warp -> block -> a max reduction on its
 // IEEE bits (non-negative doubles order like unsigned integers).
 #include <math.h>
@@ -729,6 +730,12 @@ static StepArgs make_args(const rbffd_plan* p) {
     A.fl_slot = nullptr;
     A.fl_max = 0;
     A.inner = p->inner_sl;
+    A.lk_idx = nullptr;
+    A.lk_off = nullptr;
+    A.lk_slot = nullptr;
+    A.lk_max = 0;
+    A.lk_x = A.lk_res = A.lk_dec = nullptr;
+    A.lk_epoch = 0;
     return A;
 }
 
@@ -738,6 +745,27 @@ static void far_args(const rbffd_plan* p, int mi, StepArgs* A) {
     A->fl_off = p->fl_off[mi];
     A->fl_slot = p->fl_slot[mi];
     A->fl_max = p->fl_max[mi];
+}
+
+// the linked launch's fields for a run of at most max_steps; the run takes the
+// tags of its steps.  Tags are 32 bits: before they could come round to one
+// that an old entry still carries, the entries are cleared
+static cudaError_t link_args(rbffd_plan* p, long long max_steps, StepArgs* A, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (p->lk_epoch == 0 || p->lk_epoch + (unsigned long long)max_steps + 2 > 0x80000000ull) {
+        e = cudaMemsetAsync(p->lk_x, 0, p->lk_bytes, s);
+        p->lk_epoch = 0;
+    }
+    A->lk_idx = p->lk_idx;
+    A->lk_off = p->lk_off;
+    A->lk_slot = p->lk_slot;
+    A->lk_max = p->lk_max;
+    A->lk_x = p->lk_x;
+    A->lk_res = p->lk_x + (size_t)LINK_RING * 2 * p->NI;
+    A->lk_dec = A->lk_res + (size_t)LINK_RING * 2 * p->lk_grid;
+    A->lk_epoch = (unsigned)p->lk_epoch;
+    p->lk_epoch += (unsigned long long)std::min<long long>(max_steps, 0x80000000ll) + 2;
+    return e;
 }
 
 static void drop_graphs(rbffd_plan* p) {
@@ -755,7 +783,8 @@ static void free_plan(rbffd_plan* p) {
                     p->fs, p->e[0], p->e[1], p->d32, p->scratch, p->ctrl, p->nslot, p->ncol,
                     p->nw, p->ng, p->ng0, p->uN, p->col16, p->sbase,
                     p->fl_idx[0], p->fl_idx[1], p->fl_off[0], p->fl_off[1],
-                    p->fl_slot[0], p->fl_slot[1], p->inner_sl};
+                    p->fl_slot[0], p->fl_slot[1], p->inner_sl, p->lk_idx, p->lk_off, p->lk_slot,
+                    p->lk_x};
     for (void* b : bufs)
         if (b) cudaFree(b);
     drop_graphs(p);
@@ -976,6 +1005,94 @@ static int build_far(rbffd_plan* p, int mode, cudaStream_t s) {
     return RBFFD_OK;
 }
 
+// Halo lists and local indices of the linked launch (step_link.cuh), for both
+// arithmetics: block b of G owns slices [nslices b / G, nslices (b+1) / G); the
+// slots outside its rows that its rows read go, ascending, into its list (the
+// boundary's, which follow the interior's, last), and every entry gets its
+// place: its row in the block, or the block's padded row count plus its place
+// in the list.  lk_ok stays false where the planes do not fit shared memory.
+static int build_link(rbffd_plan* p, cudaStream_t s) {
+    if (p->lk_built) return RBFFD_OK;
+    p->lk_built = true;
+    const int64_t NI = p->NI, N = p->N, nsl = p->nslices;
+    const int n = p->n;
+    const int G = (int)std::min<int64_t>(device_sm_count(), nsl);
+    int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return RBFFD_OK;
+    }
+    if (link_smem(nsl, n, MODE_INNER32, G, 0) + 1024u > (unsigned)optin) return RBFFD_OK;
+    const int64_t ent = nsl * n * SLICE;
+    std::vector<int32_t> col(ent);
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(col.data(), p->col, sizeof(int32_t) * ent,
+                                     cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
+    std::vector<uint16_t> lidx(ent, 0);
+    std::vector<int32_t> off(G + 1, 0), slots, place(N, -1);
+    int64_t most = 0;
+    for (int b = 0; b < G; ++b) {
+        const int64_t s0 = nsl * b / G, s1 = nsl * (b + 1) / G;
+        const int64_t r0 = s0 * SLICE, r1 = std::min<int64_t>(s1 * SLICE, NI);
+        const int64_t rows = (s1 - s0) * SLICE;
+        const size_t first = slots.size();
+        for (int64_t sl = s0; sl < s1; ++sl) {
+            const int lanes = (int)std::min<int64_t>(SLICE, NI - sl * SLICE);
+            for (int j = 0; j < n; ++j)
+                for (int l = 0; l < lanes; ++l) {
+                    const int32_t c = col[(sl * n + j) * SLICE + l];
+                    if ((c < r0 || c >= r1) && place[c] < 0) {
+                        place[c] = 0;
+                        slots.push_back(c);
+                    }
+                }
+        }
+        std::sort(slots.begin() + first, slots.end());
+        const int64_t nh = (int64_t)(slots.size() - first);
+        if (rows + nh > 65535) return RBFFD_OK;
+        most = std::max(most, nh);
+        for (int64_t i = 0; i < nh; ++i) place[slots[first + i]] = (int32_t)(rows + i);
+        for (int64_t sl = s0; sl < s1; ++sl) {
+            const int lanes = (int)std::min<int64_t>(SLICE, NI - sl * SLICE);
+            for (int j = 0; j < n; ++j)
+                for (int l = 0; l < lanes; ++l) {
+                    const int64_t e = (sl * n + j) * SLICE + l;
+                    const int32_t c = col[e];
+                    lidx[e] = (uint16_t)(c >= r0 && c < r1 ? c - r0 : place[c]);
+                }
+        }
+        for (int64_t i = 0; i < nh; ++i) place[slots[first + i]] = -1;
+        off[b + 1] = (int32_t)slots.size();
+    }
+    if (slots.empty()) slots.push_back(0);
+    p->lk_bytes = sizeof(unsigned long long) *
+                  ((size_t)LINK_RING * 2 * NI + (size_t)LINK_RING * 2 * G + LINK_RING);
+    cudaError_t e = cudaMalloc((void**)&p->lk_idx, sizeof(uint16_t) * ent);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p->lk_off, sizeof(int32_t) * off.size());
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p->lk_slot, sizeof(int32_t) * slots.size());
+    if (e == cudaSuccess) e = cudaMalloc((void**)&p->lk_x, p->lk_bytes);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(p->lk_idx, lidx.data(), sizeof(uint16_t) * ent, cudaMemcpyHostToDevice,
+                            s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(p->lk_off, off.data(), sizeof(int32_t) * off.size(),
+                            cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(p->lk_slot, slots.data(), sizeof(int32_t) * slots.size(),
+                            cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    RBFFD_CHECK_CUDA(e);
+    p->lk_grid = G;
+    p->lk_max = most;
+    p->lk_ok = true;
+    return RBFFD_OK;
+}
+
+// halo slots of a block up to which the linked launch needs no rival (tune_shape)
+static constexpr int64_t LINK_ONLY = 1024;
+
 // Autotuner: time every launch shape of `mode` for a few steps on this plan's
 // own stencils (u / e buffers zeroed; dt = 0 so nothing moves) and keep the
 // fastest.  Candidates: register budget minb in {1, 2, 3, 4} x blocks per SM
@@ -994,6 +1111,7 @@ struct TuneCand {
     bool resident;   // the resident persistent launch (smem bytes, halo, threads below)
     bool far;        // ... with far lists
     bool split;      // the split persistent launch (smem bytes, threads below)
+    bool link = false;   // the linked persistent launch (smem bytes, threads below)
     int threads;
     unsigned smem;
     int64_t halo;
@@ -1023,9 +1141,62 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
     const bool only_res = (p->flags & RBFFD_LAUNCH_RESIDENT) != 0 || only_far || only_split;
     const int c_lo = may_graph(p) ? 1 : 5, c_hi = may_persist(p) ? 5 : 4;
     std::vector<TuneCand> cands;
+    bool res_any = false;
+    // the linked launch, wherever the resident one may be chosen (not when
+    // rbffd_plan_set_resident_halo fixed a reach: that asks for its window).
+    // Where no block reads more than LINK_ONLY slots of others it is taken
+    // without timing the other launches: measured from 1.5k to 89k rows, n = 12 to
+    // 70, 2D and 3D, Morton and random orders, the best of them took 1.13 to 2.5
+    // times as long; above (a random order of 3D supports: 2,500 slots) it may lose
+    // (5.8 us against 5.6).
+    bool link_only = false;
+    if (may_persist(p) && !only_split && !only_far &&
+        (p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_RESIDENT)) && p->res_halo_set < -1) {
+        int st0 = build_link(p, s);
+        if (st0) return st0;
+        int dev = 0, optin = 0;
+        for (int wide = 0; wide < 2 && p->lk_ok; ++wide) {
+            TuneCand t;
+            t.threads = wide ? RES_THREADS_WIDE : RES_THREADS_HOST;
+            if (p->res_threads_set && t.threads != p->res_threads_set) continue;
+            t.fn = pick_link(mode, p->n, t.threads);
+            if (!t.fn) continue;
+            t.smem = link_smem(p->nslices, p->n, mode, p->lk_grid, p->lk_max);
+            int per_sm = 0;
+            if (cudaGetDevice(&dev) != cudaSuccess ||
+                cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+                    cudaSuccess ||
+                t.smem + 1024u > (unsigned)optin ||
+                cudaFuncSetAttribute((const void*)t.fn,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)t.smem) != cudaSuccess ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)t.fn,
+                                                              t.threads, t.smem) !=
+                    cudaSuccess ||
+                per_sm < 1) {
+                cudaGetLastError();
+                continue;
+            }
+            t.minb = 1;
+            t.pdl = false;
+            t.per_sm = 1;
+            t.persistent = true;
+            t.resident = true;
+            t.far = false;
+            t.split = false;
+            t.link = true;
+            t.halo = 0;
+            t.grid = p->lk_grid;
+            t.gx = nullptr;
+            t.ms = 1e30f;
+            res_any = true;
+            link_only = link_only || p->lk_max <= LINK_ONLY;
+            cands.push_back(t);
+        }
+    }
     const int pdl_lo = (p->flags & RBFFD_LAUNCH_PDL) ? 1 : 0;
     const int pdl_hi = (p->flags & RBFFD_LAUNCH_NO_PDL) ? 1 : 2;
-    for (int minb = 1; minb <= n_minb && !only_res; ++minb)
+    for (int minb = 1; minb <= n_minb && !only_res && !link_only; ++minb)
         for (int c = c_lo; c <= c_hi; ++c)
             for (int pdl = c == 5 ? 0 : pdl_lo; pdl < (c == 5 ? 1 : pdl_hi); ++pdl) {
                 TuneCand t;
@@ -1049,8 +1220,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
     // and the plan's planes fit one block per SM; its halo reach is tuned: no
     // window, the block's own rows, 256, 1024, 4096 slots, the most that fits;
     // and its block size: 512 threads, and 1024 where the stencil size has it
-    bool res_any = false;
-    for (int wide = 0; wide < 2 && may_persist(p) && !only_far && !only_split &&
+    for (int wide = 0; wide < 2 && may_persist(p) && !only_far && !only_split && !link_only &&
                        (p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_RESIDENT));
          ++wide) {
         TuneCand t;
@@ -1086,7 +1256,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
     }
     // the resident launch with far lists (its reach fixed by the build; not
     // when rbffd_plan_set_resident_halo fixed one)
-    if (may_persist(p) && !only_split &&
+    if (may_persist(p) && !only_split && !link_only &&
         (p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_RESIDENT | RBFFD_LAUNCH_FAR)) &&
         p->res_halo_set < -1) {
         int st0 = build_far(p, mode, s);
@@ -1128,7 +1298,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
     // the split launch: Morton plans ordered with each share's inner rows first
     // (plan creation), when its own-row buffers fit one block per SM
     bool split_any = false;
-    for (int wide = 0; wide < 2 && may_persist(p) && p->inner_first &&
+    for (int wide = 0; wide < 2 && may_persist(p) && p->inner_first && !link_only &&
                        (p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_PERSISTENT | RBFFD_LAUNCH_SPLIT));
          ++wide) {
         TuneCand t;
@@ -1218,6 +1388,11 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
                 StepCtrl* c = p->ctrl;
                 A.halo = t.halo;
                 far_args(p, mi, &A);
+                if (t.link && link_args(p, reps, &A, s) != cudaSuccess) {
+                    set_error("autotune: clearing the linked launch's entries failed");
+                    st = RBFFD_ERR_CUDA;
+                    break;
+                }
                 void* args[] = {(void*)&A, (void*)&c};
                 cudaLaunchCooperativeKernel((const void*)t.fn, dim3(t.grid),
                                             dim3(t.resident || t.split ? t.threads : STEP_THREADS),
@@ -1255,6 +1430,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
     p->res_threads[mi] = best->resident || best->split ? best->threads : RES_THREADS_HOST;
     p->res_far[mi] = best->resident && best->far;
     p->split[mi] = best->split;
+    p->link[mi] = best->link;
     p->res_halo[mi] = best->halo;
     p->tune_ms[mi] = best->ms / (float)reps;
     p->tuned[mi] = true;
@@ -1354,16 +1530,20 @@ static int run_steps(rbffd_plan* p, int mode, double dt, double tol, long long m
             // resident and split launches: one block of res_threads per SM
             const bool res = p->resident[mi] || p->split[mi];
             StepFn fn = p->split[mi] ? pick_split(mode, p->n, p->res_threads[mi])
+                        : p->link[mi] ? pick_link(mode, p->n, p->res_threads[mi])
                         : p->resident[mi]
                             ? (p->res_far[mi] ? pick_resident_far(mode, p->n, p->res_threads[mi])
                                : p->res_threads[mi] == RES_THREADS_WIDE
                                    ? pick_resident_wide(mode, p->n, res_i16(p))
                                    : pick_resident(mode, p->n, res_i16(p)))
                             : pick(mode, p->n, true, p->minb[mi]);
-            int grid = res ? device_sm_count() : persistent_grid(fn, p);
+            int grid = p->link[mi] ? p->lk_grid
+                       : res       ? device_sm_count()
+                                   : persistent_grid(fn, p);
             StepArgs A = make_args(p);
             A.halo = p->resident[mi] ? p->res_halo[mi] : 0;
             far_args(p, mi, &A);
+            if (p->link[mi]) RBFFD_CHECK_CUDA(link_args(p, max_steps, &A, s));
             StepCtrl* c = p->ctrl;
             void* args[] = {(void*)&A, (void*)&c};
             RBFFD_CHECK_CUDA(cudaEventRecord((cudaEvent_t)p->ev[0], s));
@@ -1839,7 +2019,7 @@ extern "C" int rbffd_plan_set_dc(rbffd_plan* p, int64_t K_in, double rho_in) {
 static void retune(rbffd_plan* p) {
     for (int mi = 0; mi < 2; ++mi) {
         p->tuned[mi] = false;
-        p->persist[mi] = p->resident[mi] = p->split[mi] = false;
+        p->persist[mi] = p->resident[mi] = p->split[mi] = p->link[mi] = false;
     }
     drop_graphs(p);
 }
@@ -2133,7 +2313,8 @@ extern "C" int rbffd_plan_stats(const rbffd_plan* p, double* h_loop_ms, int64_t*
     if (h_launches) *h_launches = p->last_launches;
     if (h_shape) {
         for (int mi = 0; mi < 2; ++mi) {
-            h_shape[2 * mi] = p->resident[mi] ? p->res_threads[mi] / 512 + (p->res_far[mi] ? 4 : 0)
+            h_shape[2 * mi] = p->resident[mi] ? p->res_threads[mi] / 512 + (p->res_far[mi] ? 4 : 0) +
+                                                   (p->link[mi] ? 8 : 0)
                               : p->split[mi] ? p->res_threads[mi] / 512
                                              : p->minb[mi];
             h_shape[2 * mi + 1] = p->persist[mi]

@@ -1,0 +1,102 @@
+"""The linked launch (blocks exchange rows and decisions through tagged words, no grid barrier)
+against graph-replayed steps, bit for bit, and against its own stop rule: shares of one, two and
+more slices than warps, fewer slices than SMs, one partial slice, every way a run can end and
+how many steps after the start, both block sizes, both arithmetics, and tags that start over."""
+import numpy as np
+import pytest
+
+import rbffd_inputs as gen
+from oracle_problem import build
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module")
+def rb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2502_12878_gb300 import build as nvbuild
+    nvbuild.build()
+    import paper_2502_12878_gb300 as m
+    m.lib()
+    return m
+
+
+def T(x):
+    return torch.from_numpy(np.ascontiguousarray(x)).to(DEV)
+
+
+def _plans(rb, p, threads, order=0):
+    ref = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w), order, 3)
+    lnk = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w),
+                  order | rb.RBFFD_LAUNCH_RESIDENT, 3)
+    lnk.set_block(threads)
+    return ref, lnk
+
+
+def _linked(shape):
+    return shape[1] == -1 and shape[0] >= 8
+
+
+# d, Kg, m, n, order: 9 rows; 2 blocks of one slice; fewer slices than SMs; 2-3 slices a block;
+# 8; 18 (more than 512 threads have warps for); 3D; a random order (every support scattered)
+CASES = [(2, 4, 1, 6, 0), (2, 9, 2, 12, 0), (2, 60, 2, 13, 0), (2, 100, 2, 12, 0),
+         (2, 200, 4, 30, 0), (2, 300, 4, 30, 0), (2, 120, 6, 56, 0), (3, 22, 4, 70, 0),
+         (2, 90, 2, 17, 0), (2, 70, 4, 31, 2)]
+
+
+@pytest.mark.parametrize("threads", [512, 1024])
+@pytest.mark.parametrize("d,Kg,m,n,order", CASES)
+def test_same_bits_as_graph_steps(rb, orc, d, Kg, m, n, order, threads):
+    p = build(orc, d, Kg, m, seed=7, n=n)
+    ref, lnk = _plans(rb, p, threads, order)
+    f, u0 = T(p.f), T(p.u0)
+    dt = 0.5 * 2.0 / np.abs(p.w).sum(1).max()
+    try:
+        lnk.solve_explicit(f, u0.clone(), dt, 1)
+    except rb.RbffdError as e:     # a block size not compiled for this n
+        assert e.code == rb.RBFFD_ERR_CAPACITY and threads == 1024
+        return
+    for K in (1, 2, 5, 6, 7, 40, 333):
+        a, b = u0.clone(), u0.clone()
+        ra = ref.solve_explicit(f, a, dt, K)
+        rl = lnk.solve_explicit(f, b, dt, K)
+        assert ra == rl and torch.equal(a, b), K
+    # stops by tolerance: at the first step, within and beyond the steps a block may be ahead
+    hist = []
+    u = u0.clone()
+    for k in range(12):
+        hist.append(ref.solve_explicit(f, u, dt, 1)[2])
+    for k in (0, 1, 3, 4, 5, 6, 9, 11):
+        tol = np.nextafter(hist[k], np.inf)
+        a, b = u0.clone(), u0.clone()
+        ra = ref.solve_explicit(f, a, dt, 5_000_000_000 if k == 9 else 200, tol)
+        rl = lnk.solve_explicit(f, b, dt, 5_000_000_000 if k == 9 else 200, tol)
+        assert ra == rl and torch.equal(a, b), k
+    # defect correction: FP32 inner steps, stopped by the cap and by rho_in
+    for K_in, rho in ((7, 0.0), (400, 0.9)):
+        a, b = u0.clone(), u0.clone()
+        ra = ref.solve_dc(f, a, dt, 1e-12, 3, K_in, rho)
+        rl = lnk.solve_dc(f, b, dt, 1e-12, 3, K_in, rho)
+        assert ra == rl and torch.equal(a, b)
+    assert _linked(lnk.stats()[3]) or threads == 512 and n >= 56
+
+
+def test_nonfinite_and_diverging_runs_end(rb, orc):
+    p = build(orc, 2, 80, 2, seed=9)
+    ref, lnk = _plans(rb, p, 0)
+    dt = 0.5 * 2.0 / np.abs(p.w).sum(1).max()
+    bad = p.f.copy()
+    bad[1234] = np.nan
+    for plan in (ref, lnk):
+        with pytest.raises(rb.RbffdError) as e:
+            plan.solve_explicit(T(bad), T(p.u0), dt, 100)
+        assert e.value.code == rb.RBFFD_ERR_NONFINITE
+        with pytest.raises(rb.RbffdError) as e:
+            plan.solve_explicit(T(p.f), T(p.u0), 60 * dt, 4000)
+        assert e.value.code == rb.RBFFD_ERR_DIVERGED
+    a, b = T(p.u0), T(p.u0)      # and the plan solves on
+    assert ref.solve_explicit(T(p.f), a, dt, 50) == lnk.solve_explicit(T(p.f), b, dt, 50)
+    assert torch.equal(a, b)
