@@ -26,6 +26,20 @@ int device_sm_count() {
     return sms > 0 ? sms : 1;
 }
 
+cudaError_t allow_smem(const void* fn, size_t bytes) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess) return e;
+    const int most = optin - (int)a.sharedSizeBytes;
+    if (bytes > (size_t)std::max(0, most)) return cudaErrorInvalidValue;
+    if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // ------------------------------------------------------------------- scans
 static constexpr int SCAN_THREADS = 256;
 static constexpr int SCAN_PER_THREAD = 8;

@@ -39,6 +39,12 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 
 int device_sm_count();
 
+// Lets launches of kernel fn take `bytes` of dynamic shared memory (an error
+// when a block cannot have them).  The limit is a property of the kernel, not
+// of a launch, and plans of different sizes share kernels: it is raised to the
+// most the device gives, never to what one plan needs.
+cudaError_t allow_smem(const void* fn, size_t bytes);
+
 // --------------------------------------------------- stream-ordered scratch
 // RAII holder for cudaMallocAsync memory; freed on the same stream.
 struct Scratch {

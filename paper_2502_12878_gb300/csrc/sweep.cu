@@ -882,8 +882,7 @@ static StepFn resident_fn(rbffd_plan* p, int mode, int threads, unsigned* smem, 
     StepFn fn = threads == RES_THREADS_WIDE ? pick_resident_wide(mode, p->n, i16)
                                             : pick_resident(mode, p->n, i16);
     if (!fn) return nullptr;
-    if (cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bytes) != cudaSuccess ||
+    if (allow_smem((const void*)fn, bytes) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, threads,
                                                       bytes) != cudaSuccess ||
         per_sm < 1) {
@@ -1167,9 +1166,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
                 cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
                     cudaSuccess ||
                 t.smem + 1024u > (unsigned)optin ||
-                cudaFuncSetAttribute((const void*)t.fn,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)t.smem) != cudaSuccess ||
+                allow_smem((const void*)t.fn, t.smem) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)t.fn,
                                                               t.threads, t.smem) !=
                     cudaSuccess ||
@@ -1270,9 +1267,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
             t.smem = resident_smem(p->nslices, p->n, mode, true, device_sm_count(),
                                    p->fl_halo[mi], p->fl_max[mi]);
             int per_sm = 0;
-            if (cudaFuncSetAttribute((const void*)t.fn,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)t.smem) != cudaSuccess ||
+            if (allow_smem((const void*)t.fn, t.smem) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)t.fn,
                                                               t.threads, t.smem) !=
                     cudaSuccess ||
@@ -1313,8 +1308,7 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
             cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
                 cudaSuccess ||
             t.smem + 1024u > (unsigned)optin ||
-            cudaFuncSetAttribute((const void*)t.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)t.smem) != cudaSuccess ||
+            allow_smem((const void*)t.fn, t.smem) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)t.fn, t.threads,
                                                           t.smem) != cudaSuccess ||
             per_sm < 1) {
@@ -1658,8 +1652,7 @@ extern "C" int rbffd_apply(const double* w, const int32_t* idx, int64_t nc, int 
         (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(idx)) % 16 == 0) {
         const void* fn = n % 2 ? (const void*)apply_tiles<1> : (const void*)apply_tiles<2>;
         if (smem > 48 * 1024)
-            RBFFD_CHECK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem));
+            RBFFD_CHECK_CUDA(allow_smem(fn, smem));
         const int64_t ntiles = (nc + SLICE - 1) / SLICE;
         const int64_t per_sm = std::min<int64_t>(32, (227 * 1024) / (int64_t)(smem + 1024));
         const int64_t grid =

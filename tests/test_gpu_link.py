@@ -100,3 +100,27 @@ def test_nonfinite_and_diverging_runs_end(rb, orc):
     a, b = T(p.u0), T(p.u0)      # and the plan solves on
     assert ref.solve_explicit(T(p.f), a, dt, 50) == lnk.solve_explicit(T(p.f), b, dt, 50)
     assert torch.equal(a, b)
+
+
+def test_plans_of_different_sizes_share_kernels(rb, orc):
+    """A launch's dynamic shared memory is limited by an attribute of the kernel: a smaller
+    plan tuned later must not lower it below what a larger plan of the same kernel needs."""
+    sizes = {rb.RBFFD_LAUNCH_RESIDENT: (200, 90), rb.RBFFD_LAUNCH_FAR: (180, 90),
+             rb.RBFFD_LAUNCH_SPLIT: (330, 110)}
+    for flag, kgs in sizes.items():
+        plans = []
+        for kg in kgs:
+            xyz, bnd = rb.rbffd_nodes(2, 0, kg, 0.3, 5)
+            inter = rb.rbffd_interior(bnd)
+            idx = rb.rbffd_knn(xyz, inter, 30)
+            w, _ = rb.rbffd_weights(xyz, idx, 4)
+            f = torch.ones(inter.numel(), dtype=torch.float64, device=DEV)
+            u = torch.zeros(xyz.shape[1], dtype=torch.float64, device=DEV)
+            dt = 0.5 * 2.0 / float(w.abs().sum(1).max())
+            plan = rb.Plan(xyz, bnd, inter, idx, w, flag)
+            plan.solve_explicit(f, u.clone(), dt, 3)
+            plans.append((plan, f, u, dt))
+        for plan, f, u, dt in plans + plans[::-1]:
+            a = u.clone()
+            assert plan.solve_explicit(f, a, dt, 20)[1] == 20
+            assert torch.isfinite(a).all()
