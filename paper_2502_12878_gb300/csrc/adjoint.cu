@@ -14,10 +14,11 @@
 // offset from the window's base in 13..0), which the reverse step reads
 // instead of the int32 row: 10 bytes per entry instead of 12.
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 
-#include "plan.cuh"
+#include "step.cuh"
 
 namespace rbffd {
 
@@ -483,68 +484,114 @@ __global__ void adj_outputs(const double* S, const double* lam, const int32_t* r
 }
 
 // replay of one forward step (Eq. 6) from uin to uout, both in slot order:
-// interior rows updated, boundary slots copied (the same arithmetic as the
-// forward sweep, so the replayed iterates are the forward's bit for bit)
-__global__ void __launch_bounds__(256, 4)
-replay_step(const double* __restrict__ w64, const int32_t* __restrict__ col,
-            const double* __restrict__ fs, const double* __restrict__ uin,
-            double* __restrict__ uout, int64_t NI, int64_t N, int n, double dt) {
-    constexpr int CH = 8;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        if (p >= NI) {
-            uout[p] = uin[p];
-            continue;
+// interior rows updated, boundary slots copied.  The forward sweep's row sums
+// (step.cuh: 16-bit neighbour codes, fixed lengths, loads in phases, 64
+// registers), so the replayed iterates are the forward's bit for bit, and a
+// programmatic dependent launch.  Bound like the sweep by the FP64 pipe and
+// latency; with wgrad_group's sums of whole groups a step of rbffd_adjoint_w (K = 64,
+// spacing 8) went at 9.8k rows, n = 12 from 20.8 to 10.8 us, at 89k, n = 30 from 40.8
+// to 31.7, at 1M from 267 to 209 (phases of eight over the 16-bit codes at any
+// length, in place of the fixed lengths: 48 and 312).
+template <int NN>
+__global__ void __launch_bounds__(STEP_THREADS, 4)
+replay_step(StepArgs A, const double* __restrict__ uin, double* __restrict__ uout, double dt) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (STEP_THREADS / 32);
+    for (int64_t sl = step_warp(A); sl < A.nslices; sl += nw) {
+        const int64_t row = sl * SLICE + lane;
+        const int64_t base = sl * (int64_t)A.n * SLICE + lane;
+        if (row < A.NI) {
+            const int4 sb = A.col16 ? __ldg(A.sbase + sl) : make_int4(-1, -1, -1, -1);
+            const double fi = ld_stream(A.f + row);
+            const double ui = ld_iter<false>(uin + row);
+            double acc = 0.0;
+            if constexpr (NN > 0) {
+                acc = sb.x >= 0 ? row_dot<NN, false, true, double>(A.w64 + base, A.col16 + base,
+                                                                   sb, uin, A.n)
+                                : row_dot64<NN>(A.w64 + base, A.col + base, uin, A.n);
+            } else {   // phases of eight, which fit the budget for any n
+                constexpr int CH = 8;
+                for (int j0 = 0; j0 < A.n; j0 += CH) {
+                    int32_t c[CH];
+                    double wv[CH], uv[CH];
+#pragma unroll
+                    for (int t = 0; t < CH; ++t)
+                        if (j0 + t < A.n) c[t] = ld_stream(A.col + base + (j0 + t) * SLICE);
+#pragma unroll
+                    for (int t = 0; t < CH; ++t)
+                        if (j0 + t < A.n) wv[t] = ld_stream(A.w64 + base + (j0 + t) * SLICE);
+#pragma unroll
+                    for (int t = 0; t < CH; ++t)
+                        if (j0 + t < A.n) uv[t] = ld_iter<false>(uin + c[t]);
+#pragma unroll
+                    for (int t = 0; t < CH; ++t)
+                        if (j0 + t < A.n) acc = __fma_rn(wv[t], uv[t], acc);
+                }
+            }
+            uout[row] = __fma_rn(dt, __dsub_rn(acc, fi), ui);
         }
-        const int64_t base = (p / SLICE) * (int64_t)n * SLICE + (p % SLICE);
-        double acc = 0.0;
-        for (int j0 = 0; j0 < n; j0 += CH) {
-            int32_t c[CH];
-            double wv[CH], uv[CH];
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) c[t] = adj_ld_cs(col + base + (int64_t)(j0 + t) * SLICE);
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) wv[t] = adj_ld_cs(w64 + base + (int64_t)(j0 + t) * SLICE);
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) uv[t] = adj_ld_nc(uin + c[t]);
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) acc = __fma_rn(wv[t], uv[t], acc);
-        }
-        double r = __dsub_rn(acc, fs[p]);
-        uout[p] = __fma_rn(dt, r, uin[p]);
     }
+    for (int64_t p = A.NI + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < A.N;
+         p += (int64_t)gridDim.x * blockDim.x)
+        uout[p] = uin[p];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// weight-gradient accumulation with lambda^{k+1} and u^k in the slice layout:
-// G[s][j][lane] = fma(lambda_p, u^k[col], G[s][j][lane])
-__global__ void __launch_bounds__(256, 4)
-wgrad_accum(const int32_t* __restrict__ col, const double* __restrict__ lam,
-            const int32_t* __restrict__ posof, const double* __restrict__ uk,
-            double* __restrict__ G, int64_t NI, int n) {
-    constexpr int CH = 8;
+// weight-gradient accumulation over up to WG_STEPS steps at once, in the slice
+// layout: G[s][j][lane] = fma(lambda^{k+1}_p, u^k[col], G[s][j][lane]) for k =
+// k_hi, k_hi - 1, ..., the same chain as step by step.  One step at a time reads
+// and writes all of G (16 bytes an entry) for one multiply-add per entry;
+// together the entry's index and G are read once.  lam: the steps' lambda, newest
+// last (`lstep` entries apart, in ring order); u: u^{k_hi}, each older one N before.
+// `first`: G is not read (it is 0).  Bound by the FP64 pipe (one multiply-add per
+// entry and step) and the gathers' latency: 58 us for eight steps at 89k rows, n
+// = 30, where eight single steps took 100 (the pipe alone: 37).
+static constexpr int WG_STEPS = 8;
+
+struct LamRing {
+    const double* p[WG_STEPS];
+};
+
+template <int M>
+__global__ void __launch_bounds__(256, 3)
+wgrad_group(const int32_t* __restrict__ col, const uint16_t* __restrict__ col16,
+            const int4* __restrict__ sbase, const LamRing lam, const int32_t* __restrict__ posof,
+            const double* __restrict__ u, double* __restrict__ G, int64_t NI, int64_t N, int n,
+            bool first) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
          p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t base = (p / SLICE) * (int64_t)n * SLICE + (p % SLICE);
-        const double lp = lam[posof[p]];   // lambda is held in the placed order
+        const int4 sb = col16 ? __ldg(sbase + p / SLICE) : make_int4(-1, -1, -1, -1);
+        const int32_t pos = posof[p];   // lambda is held in the placed order
+        double l[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) l[i] = lam.p[i][pos];
+        constexpr int CH = 2;
         for (int j0 = 0; j0 < n; j0 += CH) {
             int32_t c[CH];
-            double gv[CH], uv[CH];
+            double g[CH], uv[CH][M];
+#pragma unroll
+            for (int t = 0; t < CH; ++t) {
+                const int64_t e = base + (int64_t)(j0 + t) * SLICE;
+                if (j0 + t < n) {
+                    c[t] = sb.x >= 0 ? adj_decode16(adj_ld_cs(col16 + e), sb)
+                                     : adj_ld_cs(col + e);
+                    g[t] = first ? 0.0 : G[e];
+                }
+            }
 #pragma unroll
             for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) c[t] = adj_ld_cs(col + base + (int64_t)(j0 + t) * SLICE);
+#pragma unroll
+                for (int i = 0; i < M; ++i)
+                    if (j0 + t < n) uv[t][i] = adj_ld_nc(u + c[t] - (int64_t)i * N);
 #pragma unroll
             for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) gv[t] = G[base + (int64_t)(j0 + t) * SLICE];
+                if (j0 + t < n) {
 #pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) uv[t] = adj_ld_nc(uk + c[t]);
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < n) G[base + (int64_t)(j0 + t) * SLICE] = __fma_rn(lp, uv[t], gv[t]);
+                    for (int i = 0; i < M; ++i) g[t] = __fma_rn(l[i], uv[t][i], g[t]);
+                    G[base + (int64_t)(j0 + t) * SLICE] = g[t];
+                }
         }
     }
 }
@@ -594,6 +641,44 @@ static cudaError_t adj_launch(AdjStepFn fn, unsigned grid, bool pdl, cudaStream_
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, fn, T, NI, dt, lam, lam_out, S);
+}
+
+// a kernel launch that may start while its predecessor (a kernel of the same
+// stream) drains: the kernel itself waits before it reads
+template <class... P, class... V>
+static cudaError_t launch_dependent(void (*fn)(P...), unsigned grid, unsigned threads,
+                                    cudaStream_t s, V... v) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, v...);
+}
+
+static void launch_wgrad(int m, unsigned grid, cudaStream_t s, const rbffd_plan* p,
+                         const LamRing& lam, const int32_t* posof, const double* u, double* G,
+                         bool first) {
+#define RBFFD_WG(M)                                                                              \
+    case M:                                                                                      \
+        wgrad_group<M><<<grid, 256, 0, s>>>(p->col, p->col16, p->sbase, lam, posof, u, G, p->NI, \
+                                            p->N, p->n, first);                                  \
+        break;
+    switch (m) {
+        RBFFD_WG(1)
+        RBFFD_WG(2)
+        RBFFD_WG(3)
+        RBFFD_WG(4)
+        RBFFD_WG(5)
+        RBFFD_WG(6)
+        RBFFD_WG(7)
+        RBFFD_WG(8)
+    }
+#undef RBFFD_WG
 }
 
 static unsigned adj_grid(const rbffd_plan* p) {
@@ -838,36 +923,90 @@ extern "C" int rbffd_adjoint_w(rbffd_plan* p, const double* f, const double* ckp
     const int64_t N = p->N, NI = p->NI;
     const int n = p->n;
     const int64_t seg = std::min<int64_t>(every, std::max<int64_t>(K, 1));
-    Scratch segbuf, gacc;
+    // the segment's iterates, the lambdas of up to WG_STEPS steps and the one after
+    // them (a ring), the weight gradient's accumulator
+    constexpr int RING = WG_STEPS + 1;
+    Scratch segbuf, gacc, lamring;
     RBFFD_CHECK_CUDA(segbuf.alloc(sizeof(double) * (size_t)seg * N, s));
     RBFFD_CHECK_CUDA(gacc.alloc(sizeof(double) * (size_t)p->nslices * n * SLICE, s));
+    RBFFD_CHECK_CUDA(lamring.alloc(sizeof(double) * (size_t)RING * NI, s));
     double* U = segbuf.as<double>();
     double* Gw = gacc.as<double>();
-    RBFFD_CHECK_CUDA(cudaMemsetAsync(Gw, 0, sizeof(double) * (size_t)p->nslices * n * SLICE, s));
-    // f in slot order for the replays; lambda^K in slot order
-    adj_gather<<<G, 256, 0, s>>>(f, p->row_of_slot, NI, p->fs);
-    adj_gather_placed<<<G, 256, 0, s>>>(dLdu, p->perm, T.colof, NI, T.lam[0]);
+    auto lam = [&](int i) { return lamring.as<double>() + (int64_t)(i % RING) * NI; };
+    if (K == 0)   // else the first group writes every entry
+        RBFFD_CHECK_CUDA(
+            cudaMemsetAsync(Gw, 0, sizeof(double) * (size_t)p->nslices * n * SLICE, s));
+    // f in slot order for the replays; lambda^K in placed order
     RBFFD_CHECK_CUDA(cudaMemsetAsync(T.S, 0, sizeof(double) * NI, s));
+    adj_gather<<<G, 256, 0, s>>>(f, p->row_of_slot, NI, p->fs);
+    adj_gather_placed<<<G, 256, 0, s>>>(dLdu, p->perm, T.colof, NI, lam(0));
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    StepArgs A;
+    memset(&A, 0, sizeof(A));
+    A.w64 = p->w64;
+    A.col = p->col;
+    A.col16 = p->col16;
+    A.sbase = p->sbase;
+    A.f = p->fs;
+    A.NI = NI;
+    A.N = N;
+    A.nslices = p->nslices;
+    A.n = n;
+    // fewer slices than one block of warps per SM: spread over all SMs (step_warp)
+    const int64_t full = (p->nslices + STEP_THREADS / 32 - 1) / (STEP_THREADS / 32);
+    A.spread = full < sms ? 1 : 0;
+    const unsigned rgrid = (unsigned)std::max<int64_t>(
+        1, std::min<int64_t>(A.spread ? p->nslices : full, (int64_t)sms * 4));
+    typedef void (*ReplayFn)(StepArgs, const double*, double*, double);
+    ReplayFn replay = replay_step<0>;
+#define RBFFD_REPLAY(NN) \
+    case NN: replay = replay_step<NN>; break;
+    switch (n) {   // the stencil sizes with a compiled sweep
+        RBFFD_REPLAY(6)
+        RBFFD_REPLAY(12)
+        RBFFD_REPLAY(13)
+        RBFFD_REPLAY(16)
+        RBFFD_REPLAY(20)
+        RBFFD_REPLAY(24)
+        RBFFD_REPLAY(30)
+        RBFFD_REPLAY(31)
+        RBFFD_REPLAY(40)
+        RBFFD_REPLAY(48)
+        RBFFD_REPLAY(56)
+        RBFFD_REPLAY(57)
+        RBFFD_REPLAY(70)
+        RBFFD_REPLAY(71)
+    }
+#undef RBFFD_REPLAY
     const int64_t nseg = (K + every - 1) / every;
-    const unsigned agrid = T.step_grid;
-    int cur = 0;   // lambda^{k+1} lives in T.lam[cur]
+    const unsigned wgrid =
+        (unsigned)std::max<int64_t>(1, std::min<int64_t>((NI + 255) / 256, (int64_t)sms * 24));
+    int cur = 0;   // lambda^{k+1} lives in lam(cur)
+    bool first = true;
     for (int64_t sidx = nseg - 1; sidx >= 0; --sidx) {
         const int64_t k0 = sidx * every, k1 = std::min(K, k0 + every);
         // u^{k0} from its checkpoint, then replay u^{k0+1} .. u^{k1-1}
         ckpt_gather<<<G, 256, 0, s>>>(ckpt + sidx * N, p->perm, N, U);
         for (int64_t k = k0; k + 1 < k1; ++k)
-            replay_step<<<G, 256, 0, s>>>(p->w64, p->col, p->fs, U + (k - k0) * N,
-                                          U + (k - k0 + 1) * N, NI, N, n, dt);
-        for (int64_t k = k1 - 1; k >= k0; --k) {
-            wgrad_accum<<<G, 256, 0, s>>>(p->col, T.lam[cur], T.posof, U + (k - k0) * N, Gw, NI,
-                                          n);
-            T.step<<<agrid, 256, 0, s>>>(T, NI, dt, T.lam[cur], T.lam[cur ^ 1], T.S);
-            cur ^= 1;
+            RBFFD_CHECK_CUDA(launch_dependent(replay, rgrid, STEP_THREADS, s, A,
+                                              (const double*)(U + (k - k0) * N),
+                                              U + (k - k0 + 1) * N, dt));
+        for (int64_t k = k1 - 1; k >= k0;) {
+            const int m = (int)std::min<int64_t>(WG_STEPS, k - k0 + 1);
+            LamRing ring;
+            for (int i = 0; i < WG_STEPS; ++i) ring.p[i] = lam(cur + std::min(i, m - 1));
+            for (int i = 0; i < m; ++i)
+                RBFFD_CHECK_CUDA(adj_launch(T.step, T.step_grid, T.step_pdl, s, T, NI, dt,
+                                            lam(cur + i), lam(cur + i + 1), T.S));
+            launch_wgrad(m, wgrid, s, p, ring, T.posof, U + (k - k0) * N, Gw, first);
+            first = false;
+            cur = (cur + m) % RING;
+            k -= m;
         }
         RBFFD_CHECK_CUDA(cudaGetLastError());
     }
     adjoint_grad_g<<<G, 256, 0, s>>>(T, NI, N, dt, T.S, p->perm, dLdu, grad_g);
-    adj_outputs<<<G, 256, 0, s>>>(T.S, T.lam[cur], p->row_of_slot, T.colof, p->perm, NI, dt,
+    adj_outputs<<<G, 256, 0, s>>>(T.S, lam(cur), p->row_of_slot, T.colof, p->perm, NI, dt,
                                   grad_f,
                                   grad_g, lam0);
     wgrad_unpack<<<G, 256, 0, s>>>(Gw, p->row_of_slot, NI, n, dt, grad_w);
