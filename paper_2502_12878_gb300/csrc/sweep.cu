@@ -158,44 +158,78 @@ __global__ void check_interior(const uint8_t* is_bnd, const int32_t* interior, c
 }
 
 __global__ void count_interior(const uint8_t* is_bnd, int64_t N, unsigned long long* cnt) {
-    unsigned long long c = 0;
+    __shared__ int wc[32];
+    int c = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x)
         c += is_bnd[i] ? 0 : 1;
-    atomicAdd(cnt, c);
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) wc[threadIdx.x >> 5] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {   // one atomic per block (one per thread: 200 us)
+        int t = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wc[w];
+        if (t) atomicAdd(cnt, (unsigned long long)t);
+    }
 }
 
-__global__ void pack_stencils(const int32_t* row_of_slot, const int32_t* inv, const int32_t* idx,
-                              const double* w, int64_t NI, int64_t nslices, int n, int64_t N,
-                              double* w64, float* w32, int32_t* col, int* err) {
-    const int64_t total = nslices * SLICE;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < total;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        int64_t sl = p / SLICE, lane = p % SLICE;
-        int64_t base = sl * (int64_t)n * SLICE + lane;
+// The packed planes from the caller's row-major stencils, a warp per slice:
+// each row's entries are read in memory order (a row is one contiguous run, but
+// the rows of a slice lie anywhere), up to PACK_COLS of them at a time, and
+// turned in shared memory (odd pitch) so that every plane is written as whole lines.
+// A thread per row, which read its own row one word of a sector at a time, took
+// 342 us for 1M rows, n = 30 (840 MB: 124 us), and ran twice on plans that order
+// inner rows first; this takes 258 and runs once.
+static constexpr int PACK_WARPS = 4;
+static constexpr int PACK_COLS = 16;
+
+__global__ void __launch_bounds__(32 * PACK_WARPS)
+pack_stencils(const int32_t* __restrict__ row_of_slot, const int32_t* __restrict__ inv,
+              const int32_t* __restrict__ idx, const double* __restrict__ w, int64_t NI,
+              int64_t nslices, int n, int64_t N, double* __restrict__ w64,
+              float* __restrict__ w32, int32_t* __restrict__ col, int* err) {
+    __shared__ double ws[PACK_WARPS][SLICE][PACK_COLS + 1];
+    __shared__ int32_t is[PACK_WARPS][SLICE][PACK_COLS + 1];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int half = lane >> 4, c = lane & 15;   // two rows at a time, a lane per entry
+    for (int64_t sl = (int64_t)blockIdx.x * PACK_WARPS + wib; sl < nslices;
+         sl += (int64_t)gridDim.x * PACK_WARPS) {
+        const int64_t p = sl * SLICE + lane;
         int32_t r = p < NI ? row_of_slot[p] : -1;
         if (p < NI && (r < 0 || r >= NI)) {
             atomicExch(err, 2);   // slot not covered by the interior list
             r = -1;
         }
-        if (r >= 0) {
-            for (int j = 0; j < n; ++j) {
-                int32_t nb = idx[(int64_t)r * n + j];
-                if (nb < 0 || nb >= N) {
+        const int64_t base = sl * (int64_t)n * SLICE + lane;
+        for (int j0 = 0; j0 < n; j0 += PACK_COLS) {
+            const int m = min(PACK_COLS, n - j0);
+#pragma unroll 8
+            for (int q = 0; q < SLICE; q += 2) {
+                const int32_t rq = __shfl_sync(0xffffffffu, r, q + half);
+                double wv = 0.0;
+                int32_t nb = -1;
+                if (rq >= 0 && c < m) {
+                    const int64_t e = (int64_t)rq * n + j0 + c;
+                    wv = w[e];
+                    nb = idx[e];
+                }
+                ws[wib][q + half][c] = wv;
+                is[wib][q + half][c] = nb;
+            }
+            __syncwarp();
+            for (int j = 0; j < m; ++j) {
+                const double wv = ws[wib][lane][j];
+                int32_t nb = is[wib][lane][j];
+                if (r >= 0 && (nb < 0 || nb >= N)) {
                     atomicExch(err, 3);
                     nb = 0;
                 }
-                double wv = w[(int64_t)r * n + j];
-                w64[base + j * SLICE] = wv;
-                w32[base + j * SLICE] = (float)wv;
-                col[base + j * SLICE] = inv[nb];
+                const int64_t o = base + (int64_t)(j0 + j) * SLICE;
+                w64[o] = wv;
+                w32[o] = (float)wv;
+                col[o] = r >= 0 ? inv[nb] : 0;
             }
-        } else {
-            for (int j = 0; j < n; ++j) {
-                w64[base + j * SLICE] = 0.0;
-                w32[base + j * SLICE] = 0.0f;
-                col[base + j * SLICE] = 0;
-            }
+            __syncwarp();
         }
     }
 }
@@ -1708,23 +1742,36 @@ __device__ __forceinline__ int share_of(int64_t sl, int64_t nsl, int G) {
     return (int)b;
 }
 
-// per interior slot: 1 when every neighbour slot of its row lies in its share
-__global__ void share_inner_flags(const int32_t* __restrict__ col, int64_t NI, int64_t nsl, int n,
-                                  int G, uint8_t* __restrict__ flag) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < NI;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t sl = r / SLICE;
+// per interior slot: 1 when every neighbour slot of its row lies in its share.
+// A warp per row, the row's supports read in order (from the caller's arrays, so
+// that the planes need packing only once, in the final order)
+__global__ void share_inner_flags(const int32_t* __restrict__ row_of_slot,
+                                  const int32_t* __restrict__ idx,
+                                  const int32_t* __restrict__ inv, int64_t N, int64_t NI,
+                                  int64_t nsl, int n, int G, uint8_t* __restrict__ flag) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t sl = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sl < nsl;
+         sl += nw) {
         const int b = share_of(sl, nsl, G);
         const int64_t c0 = nsl * b / G * SLICE;
         const int64_t c1e = nsl * (b + 1) / G * SLICE;
         const int64_t c1 = c1e < NI ? c1e : NI;
-        const int64_t base = sl * n * SLICE + r % SLICE;
-        bool in = true;
-        for (int j = 0; j < n && in; ++j) {
-            const int32_t c = col[base + (int64_t)j * SLICE];
-            in = c >= c0 && c < c1;
+        const int64_t p = sl * SLICE + lane;
+        const int32_t r = p < NI ? row_of_slot[p] : -1;
+        unsigned inner = 0;
+        for (int q = 0; q < SLICE; ++q) {
+            const int32_t rq = __shfl_sync(0xffffffffu, r, q);
+            bool in = true;
+            if (rq >= 0 && rq < NI)   // (others are reported by the packing)
+                for (int j = lane; j < n; j += 32) {
+                    const int32_t nb = idx[(int64_t)rq * n + j];
+                    const int32_t s = nb >= 0 && nb < N ? inv[nb] : -1;
+                    in = in && s >= c0 && s < c1;
+                }
+            if (__all_sync(0xffffffffu, in)) inner |= 1u << q;
         }
-        flag[r] = in ? 1 : 0;
+        if (p < NI) flag[p] = (inner >> lane) & 1u;
     }
 }
 
@@ -1901,8 +1948,31 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
             break;
         check_interior<<<G, 256, 0, s>>>(is_bnd, interior, p->inv, N, NI, p->row_of_slot,
                                          err.as<int>());
-        pack_stencils<<<G, 256, 0, s>>>(p->row_of_slot, p->inv, idx, w, NI, p->nslices, n, N,
-                                        p->w64, p->w32, p->col, err.as<int>());
+        if (inner_first_applies(p, flags)) {
+            // on the device: each row's flag, then per share a stable partition
+            // of its slots (perm copied to `key` first)
+            Scratch fl;
+            if ((e = fl.alloc(NI, s)) != cudaSuccess) break;
+            if ((e = cudaMalloc((void**)&p->inner_sl, sizeof(int32_t) * sms)) != cudaSuccess) break;
+            share_inner_flags<<<G, 256, 0, s>>>(p->row_of_slot, idx, p->inv, N, NI, p->nslices, n,
+                                                sms, fl.as<uint8_t>());
+            if ((e = cudaMemcpyAsync(key.p, p->perm, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice,
+                                     s)) != cudaSuccess)
+                break;
+            share_partition<<<sms, 1024, 0, s>>>(fl.as<uint8_t>(), key.as<int32_t>(), p->perm, NI,
+                                                 p->nslices, sms, p->inner_sl);
+            p->inner_first = true;
+            invert_perm<<<G, 256, 0, s>>>(p->perm, N, p->inv);
+            if ((e = cudaMemsetAsync(p->row_of_slot, 0xff, sizeof(int32_t) * NI, s)) !=
+                cudaSuccess)
+                break;
+            check_interior<<<G, 256, 0, s>>>(is_bnd, interior, p->inv, N, NI, p->row_of_slot,
+                                             err.as<int>());
+        }
+        pack_stencils<<<(unsigned)std::min<int64_t>((p->nslices + PACK_WARPS - 1) / PACK_WARPS,
+                                                    (int64_t)sms * 8),
+                        32 * PACK_WARPS, 0, s>>>(p->row_of_slot, p->inv, idx, w, NI, p->nslices,
+                                                 n, N, p->w64, p->w32, p->col, err.as<int>());
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         unsigned long long hv[2] = {0, 0};
         if ((e = cudaMemcpyAsync(hv, err.p, sizeof(hv), cudaMemcpyDeviceToHost, s)) !=
@@ -1917,38 +1987,6 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
                                   "exactly once (NI = number of interior nodes)");
             st = RBFFD_ERR_ARG;
             break;
-        }
-        if (inner_first_applies(p, flags)) {
-            // on the device: each row's flag, then per share a stable partition
-            // of its slots (perm copied to `key` first)
-            Scratch fl;
-            if ((e = fl.alloc(NI, s)) != cudaSuccess) break;
-            if ((e = cudaMalloc((void**)&p->inner_sl, sizeof(int32_t) * sms)) != cudaSuccess) break;
-            share_inner_flags<<<G, 256, 0, s>>>(p->col, NI, p->nslices, n, sms, fl.as<uint8_t>());
-            if ((e = cudaMemcpyAsync(key.p, p->perm, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice,
-                                     s)) != cudaSuccess)
-                break;
-            share_partition<<<sms, 1024, 0, s>>>(fl.as<uint8_t>(), key.as<int32_t>(), p->perm, NI,
-                                                 p->nslices, sms, p->inner_sl);
-            p->inner_first = true;
-            invert_perm<<<G, 256, 0, s>>>(p->perm, N, p->inv);
-            if ((e = cudaMemsetAsync(p->row_of_slot, 0xff, sizeof(int32_t) * NI, s)) !=
-                cudaSuccess)
-                break;
-            check_interior<<<G, 256, 0, s>>>(is_bnd, interior, p->inv, N, NI, p->row_of_slot,
-                                             err.as<int>());
-            pack_stencils<<<G, 256, 0, s>>>(p->row_of_slot, p->inv, idx, w, NI, p->nslices, n, N,
-                                            p->w64, p->w32, p->col, err.as<int>());
-            if ((e = cudaGetLastError()) != cudaSuccess) break;
-            if ((e = cudaMemcpyAsync(hv, err.p, sizeof(hv), cudaMemcpyDeviceToHost, s)) !=
-                    cudaSuccess ||
-                (e = cudaStreamSynchronize(s)) != cudaSuccess)
-                break;
-            if (hv[0] & 0xffffffffull) {
-                set_error("rbffd_plan_create: repacking the resident shares failed");
-                st = RBFFD_ERR_CUDA;
-                break;
-            }
         }
         if (!(flags & RBFFD_PACK_IDX32)) {
             if ((e = cudaMalloc((void**)&p->col16, sizeof(uint16_t) * ell)) != cudaSuccess) break;
