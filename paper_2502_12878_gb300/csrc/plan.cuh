@@ -50,6 +50,7 @@ struct rbffd_plan {
     int n = 0;
     int flags = 0;
     int64_t nslices = 0;
+    void* slab = nullptr;           // the arrays made at creation, one allocation:
     int32_t* perm = nullptr;        // [N] slot -> original node
     int32_t* inv = nullptr;         // [N] original node -> slot
     int32_t* row_of_slot = nullptr; // [NI] slot -> row of the caller's interior list

@@ -32,6 +32,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "step.cuh"
@@ -813,12 +814,14 @@ static void drop_graphs(rbffd_plan* p) {
 
 static void free_plan(rbffd_plan* p) {
     if (!p) return;
-    void* bufs[] = {p->perm, p->inv, p->row_of_slot, p->w64, p->w32, p->col, p->u[0], p->u[1],
-                    p->fs, p->e[0], p->e[1], p->d32, p->scratch, p->ctrl, p->nslot, p->ncol,
-                    p->nw, p->ng, p->ng0, p->uN, p->col16, p->sbase,
-                    p->fl_idx[0], p->fl_idx[1], p->fl_off[0], p->fl_off[1],
-                    p->fl_slot[0], p->fl_slot[1], p->inner_sl, p->lk_idx, p->lk_off, p->lk_slot,
-                    p->lk_x};
+    if (p->slab) {
+        // nothing on the device uses it any more (cudaFree would wait, too)
+        cudaDeviceSynchronize();
+        cudaFreeAsync(p->slab, cudaStreamPerThread);
+    }
+    void* bufs[] = {p->nslot, p->ncol, p->nw, p->ng, p->ng0, p->uN, p->fl_idx[0], p->fl_idx[1],
+                    p->fl_off[0], p->fl_off[1], p->fl_slot[0], p->fl_slot[1], p->lk_idx, p->lk_off,
+                    p->lk_slot, p->lk_x};
     for (void* b : bufs)
         if (b) cudaFree(b);
     drop_graphs(p);
@@ -1862,32 +1865,45 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
     p->nslices = (NI + SLICE - 1) / SLICE;
     p->grid_steps = 2;
     const size_t ell = (size_t)p->nslices * n * SLICE;
+    // every array of the plan in one allocation, each on a 256-byte boundary
+    const int sm_count = device_sm_count();
+    const bool inner = inner_first_applies(p, flags), codes = !(flags & RBFFD_PACK_IDX32);
     cudaError_t e = cudaSuccess;
-#define RBFFD_ALLOC(ptr, bytes) \
-    if (e == cudaSuccess) e = cudaMalloc((void**)&(ptr), (bytes));
-    RBFFD_ALLOC(p->perm, sizeof(int32_t) * N);
-    RBFFD_ALLOC(p->inv, sizeof(int32_t) * N);
-    RBFFD_ALLOC(p->row_of_slot, sizeof(int32_t) * NI);
-    RBFFD_ALLOC(p->w64, sizeof(double) * ell);
-    RBFFD_ALLOC(p->w32, sizeof(float) * ell);
-    RBFFD_ALLOC(p->col, sizeof(int32_t) * ell);
-    RBFFD_ALLOC(p->u[0], sizeof(double) * N);
-    RBFFD_ALLOC(p->u[1], sizeof(double) * N);
-    // f and d32 padded to whole slices (the resident launch copies whole slices)
-    RBFFD_ALLOC(p->fs, sizeof(double) * p->nslices * SLICE);
-    RBFFD_ALLOC(p->e[0], sizeof(float) * N);
-    RBFFD_ALLOC(p->e[1], sizeof(float) * N);
-    RBFFD_ALLOC(p->d32, sizeof(float) * p->nslices * SLICE);
-    RBFFD_ALLOC(p->scratch, sizeof(double) * (2 * NI + 4096));
-    RBFFD_ALLOC(p->ctrl, sizeof(StepCtrl));
-#undef RBFFD_ALLOC
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+        size_t used = 0;
+        auto put = [&](auto** ptr, size_t bytes) {
+            if (pass) *ptr = (std::remove_reference_t<decltype(*ptr)>)((char*)p->slab + used);
+            used += (bytes + 255) / 256 * 256;
+        };
+        put(&p->perm, sizeof(int32_t) * N);
+        put(&p->inv, sizeof(int32_t) * N);
+        put(&p->row_of_slot, sizeof(int32_t) * NI);
+        put(&p->w64, sizeof(double) * ell);
+        put(&p->w32, sizeof(float) * ell);
+        put(&p->col, sizeof(int32_t) * ell);
+        put(&p->u[0], sizeof(double) * N);
+        put(&p->u[1], sizeof(double) * N);
+        // f and d32 padded to whole slices (the resident launch copies whole slices)
+        put(&p->fs, sizeof(double) * p->nslices * SLICE);
+        put(&p->e[0], sizeof(float) * N);
+        put(&p->e[1], sizeof(float) * N);
+        put(&p->d32, sizeof(float) * p->nslices * SLICE);
+        put(&p->scratch, sizeof(double) * (2 * NI + 4096));
+        put(&p->ctrl, sizeof(StepCtrl));
+        if (inner) put(&p->inner_sl, sizeof(int32_t) * sm_count);
+        if (codes) {
+            put(&p->col16, sizeof(uint16_t) * ell);
+            put(&p->sbase, sizeof(int4) * p->nslices);
+        }
+        if (!pass) e = pool_alloc(&p->slab, used, s);
+    }
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         cudaEvent_t ev;
         e = cudaEventCreate(&ev);
         if (e == cudaSuccess) p->ev[i] = (void*)ev;
     }
     if (e != cudaSuccess) {
-        set_error("rbffd_plan_create: cudaMalloc: %s", cudaGetErrorString(e));
+        set_error("rbffd_plan_create: allocation: %s", cudaGetErrorString(e));
         free_plan(p);
         return RBFFD_ERR_CUDA;
     }
@@ -1948,12 +1964,11 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
             break;
         check_interior<<<G, 256, 0, s>>>(is_bnd, interior, p->inv, N, NI, p->row_of_slot,
                                          err.as<int>());
-        if (inner_first_applies(p, flags)) {
+        if (inner) {
             // on the device: each row's flag, then per share a stable partition
             // of its slots (perm copied to `key` first)
             Scratch fl;
             if ((e = fl.alloc(NI, s)) != cudaSuccess) break;
-            if ((e = cudaMalloc((void**)&p->inner_sl, sizeof(int32_t) * sms)) != cudaSuccess) break;
             share_inner_flags<<<G, 256, 0, s>>>(p->row_of_slot, idx, p->inv, N, NI, p->nslices, n,
                                                 sms, fl.as<uint8_t>());
             if ((e = cudaMemcpyAsync(key.p, p->perm, sizeof(int32_t) * N, cudaMemcpyDeviceToDevice,
@@ -1974,7 +1989,13 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
                         32 * PACK_WARPS, 0, s>>>(p->row_of_slot, p->inv, idx, w, NI, p->nslices,
                                                  n, N, p->w64, p->w32, p->col, err.as<int>());
         if ((e = cudaGetLastError()) != cudaSuccess) break;
-        unsigned long long hv[2] = {0, 0};
+        if (codes)
+            pack_idx16<<<G, 256, 0, s>>>(p->col, NI, p->nslices, n, p->col16, p->sbase,
+                                         err.as<unsigned long long>() + 2,
+                                         reinterpret_cast<int*>(err.as<unsigned long long>() + 3));
+        if ((e = cudaGetLastError()) != cudaSuccess) break;
+        // input errors, interior nodes, rows in compact slices, packing errors
+        unsigned long long hv[4] = {0, 0, 0, 0};
         if ((e = cudaMemcpyAsync(hv, err.p, sizeof(hv), cudaMemcpyDeviceToHost, s)) !=
             cudaSuccess)
             break;
@@ -1988,26 +2009,12 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
             st = RBFFD_ERR_ARG;
             break;
         }
-        if (!(flags & RBFFD_PACK_IDX32)) {
-            if ((e = cudaMalloc((void**)&p->col16, sizeof(uint16_t) * ell)) != cudaSuccess) break;
-            if ((e = cudaMalloc((void**)&p->sbase, sizeof(int4) * p->nslices)) != cudaSuccess)
-                break;
-            if ((e = cudaMemsetAsync(err.p, 0, 4 * sizeof(unsigned long long), s)) != cudaSuccess)
-                break;
-            pack_idx16<<<G, 256, 0, s>>>(p->col, NI, p->nslices, n, p->col16, p->sbase,
-                                         err.as<unsigned long long>() + 1, err.as<int>());
-            if ((e = cudaGetLastError()) != cudaSuccess) break;
-            if ((e = cudaMemcpyAsync(hv, err.p, sizeof(hv), cudaMemcpyDeviceToHost, s)) !=
-                cudaSuccess)
-                break;
-            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-            if (hv[0] & 0xffffffffull) {
-                set_error("rbffd_plan_create: compact index packing failed");
-                st = RBFFD_ERR_CUDA;
-                break;
-            }
-            p->rows16 = (int64_t)hv[1];
+        if (hv[3] & 0xffffffffull) {
+            set_error("rbffd_plan_create: compact index packing failed");
+            st = RBFFD_ERR_CUDA;
+            break;
         }
+        p->rows16 = (int64_t)hv[2];
     } while (0);
     if (e != cudaSuccess && st == RBFFD_OK) {
         set_error("rbffd_plan_create: %s", cudaGetErrorString(e));
