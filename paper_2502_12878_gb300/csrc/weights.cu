@@ -543,9 +543,32 @@ __device__ __forceinline__ void weights_one(const WeightArgs& A, int64_t r, doub
     } while (0);
 }
 
+// The team's stencils: tickets from a counter.  Teams do not run equally
+// fast - thirteen one-warp teams on an SM are four on one of its sub-partitions,
+// which share its FP64 pipe, and three on the others - so equal shares fixed in
+// advance leave three pipes idle while the fourth finishes: 1M stencils, s = 45
+// 94.8 -> 89.9 ms; s = 46 (twelve teams: three on each) 99.7 -> 97.9; s = 18
+// 12.3 -> 12.0.  take_ticket draws the next one (the team's first thread) and is
+// called a stencil ahead, which hides the atomic's latency; share_ticket tells the team.
+__device__ __forceinline__ long long take_ticket(unsigned long long* tickets, int tid) {
+    return tid == 0 ? (long long)atomicAdd(tickets, 1ull) : 0ll;
+}
+template <int TS>
+__device__ __forceinline__ int64_t share_ticket(long long v, int tid, int team,
+                                                long long* s_next) {
+    if constexpr (TS <= 32) {
+        return __shfl_sync(team_mask<TS>(), v, 0, TS);
+    } else {
+        // (read by all before weights_one's barriers, after which it is written again)
+        if (tid == 0) s_next[team] = v;
+        team_sync<TS>();
+        return s_next[team];
+    }
+}
+
 template <int TS, bool PW>
 __global__ void __launch_bounds__(weight_max_threads(TS))
-    weights_kernel(WeightArgs A, int teams_per_block) {
+    weights_kernel(WeightArgs A, unsigned long long* tickets) {
     extern __shared__ double wsm[];
     __shared__ double redv[W_THREADS / 32];
     __shared__ long long redk[W_THREADS / 32];
@@ -556,9 +579,14 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
     const int team = threadIdx.x / TS;
     double* G = wsm + (size_t)team * weight_team_doubles(A);
     double* xi = G + (size_t)A.s * A.pitch;
-    const int64_t teams = (int64_t)gridDim.x * teams_per_block;
-    for (int64_t r = (int64_t)blockIdx.x * teams_per_block + team; r < A.nc; r += teams)
+    __shared__ long long s_next[16];
+    long long ticket = take_ticket(tickets, tid);
+    for (;;) {
+        const int64_t r = share_ticket<TS>(ticket, tid, team, s_next);
+        if (r >= A.nc) break;
+        ticket = take_ticket(tickets, tid);
         weights_one<TS, PW>(A, r, G, xi, tid, team, redv, redk, redi, bcast, spiv);
+    }
 }
 
 // many calls in one launch: stencil number g of the concatenation belongs to
@@ -567,7 +595,7 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
 template <int TS, bool PW>
 __global__ void __launch_bounds__(weight_max_threads(TS))
     weights_multi_kernel(const WeightArgs* __restrict__ calls, const int64_t* __restrict__ off,
-                         int ncalls, int teams_per_block, int64_t team_doubles) {
+                         int ncalls, unsigned long long* tickets, int64_t team_doubles) {
     extern __shared__ double wsm[];
     __shared__ double redv[W_THREADS / 32];
     __shared__ long long redk[W_THREADS / 32];
@@ -577,9 +605,13 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
     const int tid = threadIdx.x % TS;
     const int team = threadIdx.x / TS;
     double* G = wsm + (size_t)team * (size_t)team_doubles;
+    __shared__ long long s_next[16];
     const int64_t total = off[ncalls];
-    const int64_t teams = (int64_t)gridDim.x * teams_per_block;
-    for (int64_t g = (int64_t)blockIdx.x * teams_per_block + team; g < total; g += teams) {
+    long long ticket = take_ticket(tickets, tid);
+    for (;;) {
+        const int64_t g = share_ticket<TS>(ticket, tid, team, s_next);
+        if (g >= total) break;
+        ticket = take_ticket(tickets, tid);
         int lo = 0, hi = ncalls - 1;   // last call with off <= g
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -630,8 +662,9 @@ static constexpr int W_HALF_SMAX = 32;
 
 static int weight_team_size(int s) { return s <= W_HALF_SMAX ? 16 : (s <= 48 ? 32 : 160); }
 
-typedef void (*WeightKernel)(WeightArgs, int);
-typedef void (*WeightMultiKernel)(const WeightArgs*, const int64_t*, int, int, int64_t);
+typedef void (*WeightKernel)(WeightArgs, unsigned long long*);
+typedef void (*WeightMultiKernel)(const WeightArgs*, const int64_t*, int, unsigned long long*,
+                                  int64_t);
 
 // the five-warp team has a pivot warp
 static WeightKernel weight_kernel_for(int ts) {
@@ -660,14 +693,13 @@ static cudaError_t pick_weight_shape(K kern, int ts, size_t per_team, WeightShap
     const int max_tpb = std::min(weight_max_threads(ts) / ts, 15);   // named barriers 1..15
     const int step = ts == 16 ? 2 : 1;             // whole warps
     int best = -1;
+    const cudaError_t le = allow_smem((const void*)kern, 48 * 1024);
+    if (le != cudaSuccess) return le;
     for (int tpb = step; tpb <= max_tpb; tpb += step) {
         const size_t smem = per_team * tpb;
         if (smem > 227 * 1024) break;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)std::max<size_t>(smem, 48 * 1024));
-        if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tpb * ts, smem);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, tpb * ts, smem);
         if (e != cudaSuccess) return e;
         if (per_sm * tpb > best) {
             best = per_sm * tpb;
@@ -682,8 +714,7 @@ static cudaError_t pick_weight_shape(K kern, int ts, size_t per_team, WeightShap
     b.threads = b.tpb * ts;
     b.smem = per_team * b.tpb;
     *out = b;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)std::max<size_t>(b.smem, 48 * 1024));
+    return cudaSuccess;
 }
 
 // monomial exponents of degree <= m in graded order: degree ascending, then
@@ -750,12 +781,13 @@ static int weights_impl(const double* xyz, int64_t N, int d, const int32_t* idx,
     RBFFD_CHECK_CUDA(pick_weight_shape(kern, ts, per_team, &ws));
     int64_t want = (nc + ws.tpb - 1) / ws.tpb;
     int64_t grid = std::min<int64_t>(want, (int64_t)sms * ws.per_sm);
-    kern<<<(unsigned)grid, ws.threads, ws.smem, s>>>(A, ws.tpb);
+    Scratch cnt;   // singular stencils, the first of them, the teams' tickets
+    RBFFD_CHECK_CUDA(cnt.alloc(3 * sizeof(unsigned long long), s));
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.p, 0, 3 * sizeof(unsigned long long), s));
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.as<unsigned long long>() + 1, 0xff,
+                                     sizeof(unsigned long long), s));
+    kern<<<(unsigned)grid, ws.threads, ws.smem, s>>>(A, cnt.as<unsigned long long>() + 2);
     RBFFD_CHECK_CUDA(cudaGetLastError());
-    Scratch cnt;
-    RBFFD_CHECK_CUDA(cnt.alloc(2 * sizeof(unsigned long long), s));
-    unsigned long long init[2] = {0ull, ~0ull};
-    RBFFD_CHECK_CUDA(cudaMemcpyAsync(cnt.p, init, sizeof(init), cudaMemcpyHostToDevice, s));
     count_bad<<<sms * 4, 256, 0, s>>>(status, nc, cnt.as<unsigned long long>(),
                                       cnt.as<unsigned long long>() + 1);
     RBFFD_CHECK_CUDA(cudaGetLastError());
@@ -855,9 +887,12 @@ extern "C" int rbffd_weights_batch(int ncalls, const double* const* xyz, const i
         RBFFD_CHECK_CUDA(pick_weight_shape(kern, ts, per_team, &ws));
         const int64_t want = (off.back() + ws.tpb - 1) / ws.tpb;
         const int64_t grid = std::min<int64_t>(want, (int64_t)sms * ws.per_sm);
-        kern<<<(unsigned)grid, ws.threads, ws.smem, s>>>(dcalls.as<WeightArgs>(),
-                                                         doff.as<int64_t>(), (int)sel.size(),
-                                                         ws.tpb, (int64_t)team_doubles);
+        Scratch tickets;
+        RBFFD_CHECK_CUDA(tickets.alloc(sizeof(unsigned long long), s));
+        RBFFD_CHECK_CUDA(cudaMemsetAsync(tickets.p, 0, sizeof(unsigned long long), s));
+        kern<<<(unsigned)grid, ws.threads, ws.smem, s>>>(
+            dcalls.as<WeightArgs>(), doff.as<int64_t>(), (int)sel.size(),
+            tickets.as<unsigned long long>(), (int64_t)team_doubles);
         RBFFD_CHECK_CUDA(cudaGetLastError());
     }
     // singular stencils per call
