@@ -108,10 +108,11 @@ struct rbffd_plan {
     bool lk_built = false, lk_ok = false;
     int lk_grid = 0;
     int64_t lk_max = 0;
+    void* lk_slab = nullptr;        // holds the following
     uint16_t* lk_idx = nullptr;
     int32_t* lk_off = nullptr;
     int32_t* lk_slot = nullptr;
-    unsigned long long* lk_x = nullptr;   // ring, residuals and decisions, one allocation
+    unsigned long long* lk_x = nullptr;   // ring, residuals and decisions
     size_t lk_bytes = 0;
     unsigned long long lk_epoch = 0;
     int64_t res_halo[2] = {0, 0};       // and its halo reach (slots beyond a block's rows)

@@ -160,7 +160,7 @@ __device__ __forceinline__ double row_dot64(const double* __restrict__ w,
     return row_dot<NN, COH, false, double>(w, col, none, u, n);
 }
 
-enum : int { MODE_SWEEP64 = 0, MODE_INNER32 = 1 };
+enum : int { MODE_SWEEP64 = 0, MODE_INNER32 = 1, MODE_POWER64 = 2 };
 
 struct StepArgs {
     const double* w64;
@@ -197,7 +197,7 @@ struct StepArgs {
     // largest such list, the entry ring, residual and decision words, and the
     // tag before this run's first
     const uint16_t* lk_idx;   // [nslices][n][32]
-    const int32_t* lk_off;    // [blocks + 1]
+    const int32_t* lk_off;    // [blocks][2]: a list's start and length
     const int32_t* lk_slot;
     int64_t lk_max;
     unsigned long long* lk_x;     // [LINK_RING][NI] entries of one (FP32) or two words
@@ -602,6 +602,7 @@ StepFn pick_resident_far(int mode, int n, int threads);
 // the linked launch (step_link.cu; nullptr where `threads` is not compiled for
 // n) and its dynamic shared memory for halo lists of at most `halo` slots
 StepFn pick_link(int mode, int n, int threads);
+StepFn pick_link_power(int n, int threads);   // MODE_POWER64 (step_link_pow.cu)
 unsigned link_smem(int64_t nslices, int n, int mode, int grid, int64_t halo);
 // dynamic shared memory of a resident launch of `grid` blocks whose halo
 // window reaches `halo` slots beyond each block's rows on either side, with

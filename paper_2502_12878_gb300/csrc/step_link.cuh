@@ -215,10 +215,13 @@ __device__ __forceinline__ bool link_sync_or(bool bad) {
         : "=r"(r) : "r"(bad ? 1 : 0), "n"(TC) : "memory");
     return r != 0;
 }
+// MODE_POWER64: y <- dt (W_II y) with dt an exact power of two (the power
+// iteration; boundary slots hold 0), max |y| in the residual's place.
 template <int NN, int MODE, int TH>
 __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
-    typedef typename std::conditional<MODE == MODE_SWEEP64, double, float>::type T;
-    constexpr int EW = MODE == MODE_SWEEP64 ? 2 : 1;   // words of an entry
+    constexpr bool F64 = MODE != MODE_INNER32;
+    typedef typename std::conditional<F64, double, float>::type T;
+    constexpr int EW = F64 ? 2 : 1;   // words of an entry
     constexpr int NW = TH / 32 - 1, TC = 32 * NW;      // compute warps, and their threads
     extern __shared__ __align__(128) unsigned char rsm[];
     __shared__ unsigned long long s_wm[LINK_RING * NW];
@@ -231,8 +234,8 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
     res_range(A.nslices, &s0, &s1);
     const int nsl = (int)(s1 - s0);
     const int n = NN > 0 ? NN : A.n;
-    const int h0 = A.lk_off[blockIdx.x];
-    const int nh = A.lk_off[blockIdx.x + 1] - h0;   // halo slots, the boundary's last
+    const int h0 = A.lk_off[2 * blockIdx.x];
+    const int nh = A.lk_off[2 * blockIdx.x + 1];   // halo slots, the boundary's last
     const LinkLayout L = link_layout(nsl, n, (int)sizeof(T), A.lk_max);
     T* w_s = reinterpret_cast<T*>(rsm + L.w);
     uint16_t* idx_s = reinterpret_cast<uint16_t*>(rsm + L.idx);
@@ -264,10 +267,10 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
     // while the threads load the start iterate
     if (threadIdx.x == 0) {
         const unsigned ent = (unsigned)(nsl * n * SLICE);
-        const T* wg = (MODE == MODE_SWEEP64 ? (const T*)(const void*)A.w64
+        const T* wg = (F64 ? (const T*)(const void*)A.w64
                                             : (const T*)(const void*)A.w32) +
                       s0 * (int64_t)n * SLICE;
-        const T* fg = (MODE == MODE_SWEEP64 ? (const T*)(const void*)A.f
+        const T* fg = (F64 ? (const T*)(const void*)A.f
                                             : (const T*)(const void*)A.d32) +
                       s0 * SLICE;
         const void* src[3] = {wg, A.lk_idx + s0 * (int64_t)n * SLICE, fg};
@@ -285,8 +288,8 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
                     "r"(mbar)
                     : "memory");
     }
-    T* u0 = MODE == MODE_SWEEP64 ? (T*)(void*)A.u0 : (T*)(void*)A.e0;
-    T* u1 = MODE == MODE_SWEEP64 ? (T*)(void*)A.u1 : (T*)(void*)A.e1;
+    T* u0 = F64 ? (T*)(void*)A.u0 : (T*)(void*)A.e0;
+    T* u1 = F64 ? (T*)(void*)A.u1 : (T*)(void*)A.e1;
     const long long kmax = s_max, k0 = s_k, spin = s_spin;
     const T* ustart = (k0 & 1) ? u1 : u0;
     for (int i = threadIdx.x; i < nown; i += TH) v_s[(k0 & 1) * vlen + i] = ustart[r0 + i];
@@ -329,7 +332,7 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
     const int64_t ring = EW * A.NI;                      // words of one iterate
     unsigned long long* const X = A.lk_x;
     // a row's residual as IEEE bits of its own type (widened once per step)
-    typedef typename std::conditional<MODE == MODE_SWEEP64, unsigned long long, unsigned>::type B;
+    typedef typename std::conditional<F64, unsigned long long, unsigned>::type B;
     // one slice of a step: row ls * 32 + lane
     auto row = [&](int ls, const T* vc, T* vn, unsigned long long* xn, unsigned tag, B& m) {
         const int lr = ls * SLICE + lane;
@@ -337,7 +340,10 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
         const int eo = ls * n * SLICE + lane;
         const T acc = row_dot_far<NN, T>(w_s + eo, idx_s + eo, vc, n);
         T v;
-        if constexpr (MODE == MODE_SWEEP64) {
+        if constexpr (MODE == MODE_POWER64) {
+            v = __dmul_rn(acc, dt);
+            m = max(m, abs_bits(v));
+        } else if constexpr (MODE == MODE_SWEEP64) {
             const double r = __dsub_rn(acc, f_s[lr]);
             v = __fma_rn(dt, r, vc[lr]);
             m = max(m, abs_bits(r));
@@ -399,7 +405,7 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
             row(i, vc, vn, xn, tag + 1u, m);
         }
         if (warp < nsl) {
-            if constexpr (MODE == MODE_SWEEP64) {
+            if constexpr (F64) {
                 m = link_warp_max(m);
                 if (lane == 0) s_wm[ri * NW + warp] = m;
             } else {

@@ -818,10 +818,10 @@ static void free_plan(rbffd_plan* p) {
         // nothing on the device uses it any more (cudaFree would wait, too)
         cudaDeviceSynchronize();
         cudaFreeAsync(p->slab, cudaStreamPerThread);
+        if (p->lk_slab) cudaFreeAsync(p->lk_slab, cudaStreamPerThread);
     }
     void* bufs[] = {p->nslot, p->ncol, p->nw, p->ng, p->ng0, p->uN, p->fl_idx[0], p->fl_idx[1],
-                    p->fl_off[0], p->fl_off[1], p->fl_slot[0], p->fl_slot[1], p->lk_idx, p->lk_off,
-                    p->lk_slot, p->lk_x};
+                    p->fl_off[0], p->fl_off[1], p->fl_slot[0], p->fl_slot[1]};
     for (void* b : bufs)
         if (b) cudaFree(b);
     drop_graphs(p);
@@ -1042,11 +1042,81 @@ static int build_far(rbffd_plan* p, int mode, cudaStream_t s) {
 }
 
 // Halo lists and local indices of the linked launch (step_link.cuh), for both
-// arithmetics: block b of G owns slices [nslices b / G, nslices (b+1) / G); the
-// slots outside its rows that its rows read go, ascending, into its list (the
-// boundary's, which follow the interior's, last), and every entry gets its
-// place: its row in the block, or the block's padded row count plus its place
-// in the list.  lk_ok stays false where the planes do not fit shared memory.
+// arithmetics, one block per share (block b of G owns slices [nslices b / G,
+// nslices (b+1) / G)): a bit map of the slots outside the share that its rows read,
+// whose set bits in order are the list (the boundary's slots, which follow the
+// interior's, last); every entry gets its place: its row in the share, or the
+// share's padded row count plus its slot's rank.  listed[b] = {start, length}; a
+// list longer than LINK_CAP is only counted (the plan then does without).
+static constexpr int LINK_CAP = 4096;
+static constexpr int64_t LINK_MAX_N = 800000;   // bit map and ranks in 200 KB
+
+__global__ void __launch_bounds__(1024)
+link_lists(const int32_t* __restrict__ col, int64_t NI, int64_t N, int64_t nsl, int n,
+           uint16_t* __restrict__ lidx, int32_t* __restrict__ slots,
+           int32_t* __restrict__ listed) {
+    extern __shared__ uint32_t lmap[];
+    __shared__ int s_w[32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int words = (int)((N + 31) / 32);
+    int32_t* before = reinterpret_cast<int32_t*>(lmap + words);   // set bits before each word
+    const int64_t s0 = nsl * blockIdx.x / gridDim.x, s1 = nsl * (blockIdx.x + 1) / gridDim.x;
+    const int64_t r0 = s0 * SLICE, r1 = min(s1 * SLICE, NI);
+    const int rows = (int)((s1 - s0) * SLICE);
+    const int64_t e0 = s0 * n * SLICE, e1 = s1 * n * SLICE;
+    for (int w = t; w < words; w += 1024) lmap[w] = 0u;
+    __syncthreads();
+    for (int64_t e = e0 + t; e < e1; e += 1024) {
+        // entry e: lane e % 32 of slice e / (32 n)
+        const int64_t row = e / ((int64_t)n * SLICE) * SLICE + e % SLICE;
+        const int32_t c = col[e];
+        if (row < NI && (c < r0 || c >= r1)) atomicOr(&lmap[c >> 5], 1u << (c & 31));
+    }
+    __syncthreads();
+    const int per = (words + 1023) / 1024;
+    const int w0 = min(words, t * per), w1 = min(words, w0 + per);
+    int cnt = 0;
+    for (int w = w0; w < w1; ++w) cnt += __popc(lmap[w]);
+    int x = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[wid] = x;
+    __syncthreads();
+    int pos = x - cnt, total = 0;
+    for (int w = 0; w < 32; ++w) {
+        if (w < wid) pos += s_w[w];
+        total += s_w[w];
+    }
+    int32_t* mine = slots + (int64_t)blockIdx.x * LINK_CAP;
+    for (int w = w0; w < w1; ++w) {
+        before[w] = pos;
+        for (uint32_t m = lmap[w]; m; m &= m - 1) {
+            if (pos < LINK_CAP) mine[pos] = 32 * w + __ffs(m) - 1;
+            ++pos;
+        }
+    }
+    if (t == 0) {
+        listed[2 * blockIdx.x] = blockIdx.x * LINK_CAP;
+        listed[2 * blockIdx.x + 1] = total;
+    }
+    __syncthreads();
+    for (int64_t e = e0 + t; e < e1; e += 1024) {
+        const int64_t row = e / ((int64_t)n * SLICE) * SLICE + e % SLICE;
+        const int32_t c = col[e];
+        int l = 0;
+        if (row < NI)
+            l = c >= r0 && c < r1
+                    ? (int)(c - r0)
+                    : rows + before[c >> 5] + __popc(lmap[c >> 5] & ((1u << (c & 31)) - 1u));
+        lidx[e] = (uint16_t)l;
+    }
+}
+
+// the lists, once per plan; lk_ok stays false where they, or the planes beside
+// them, do not fit
 static int build_link(rbffd_plan* p, cudaStream_t s) {
     if (p->lk_built) return RBFFD_OK;
     p->lk_built = true;
@@ -1060,70 +1130,50 @@ static int build_link(rbffd_plan* p, cudaStream_t s) {
         cudaGetLastError();
         return RBFFD_OK;
     }
-    if (link_smem(nsl, n, MODE_INNER32, G, 0) + 1024u > (unsigned)optin) return RBFFD_OK;
+    if (N > LINK_MAX_N || link_smem(nsl, n, MODE_INNER32, G, 0) + 1024u > (unsigned)optin)
+        return RBFFD_OK;
+    const size_t map = 2 * sizeof(uint32_t) * (size_t)((N + 31) / 32);
+    RBFFD_CHECK_CUDA(allow_smem((const void*)link_lists, map));
     const int64_t ent = nsl * n * SLICE;
-    std::vector<int32_t> col(ent);
-    RBFFD_CHECK_CUDA(cudaMemcpyAsync(col.data(), p->col, sizeof(int32_t) * ent,
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t b_x = sizeof(unsigned long long) *
+                       ((size_t)LINK_RING * 2 * NI + (size_t)LINK_RING * 2 * G + LINK_RING);
+    const size_t o_off = up(b_x), o_slot = o_off + up(2 * sizeof(int32_t) * G),
+                 o_idx = o_slot + up(sizeof(int32_t) * (size_t)G * LINK_CAP);
+    RBFFD_CHECK_CUDA(pool_alloc(&p->lk_slab, o_idx + sizeof(uint16_t) * ent, s));
+    char* base = (char*)p->lk_slab;
+    p->lk_x = (unsigned long long*)base;
+    p->lk_bytes = b_x;
+    p->lk_off = (int32_t*)(base + o_off);
+    p->lk_slot = (int32_t*)(base + o_slot);
+    p->lk_idx = (uint16_t*)(base + o_idx);
+    link_lists<<<G, 1024, map, s>>>(p->col, NI, N, nsl, n, p->lk_idx, p->lk_slot, p->lk_off);
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    std::vector<int32_t> listed(2 * G);
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(listed.data(), p->lk_off, sizeof(int32_t) * 2 * G,
                                      cudaMemcpyDeviceToHost, s));
     RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
-    std::vector<uint16_t> lidx(ent, 0);
-    std::vector<int32_t> off(G + 1, 0), slots, place(N, -1);
-    int64_t most = 0;
-    for (int b = 0; b < G; ++b) {
-        const int64_t s0 = nsl * b / G, s1 = nsl * (b + 1) / G;
-        const int64_t r0 = s0 * SLICE, r1 = std::min<int64_t>(s1 * SLICE, NI);
-        const int64_t rows = (s1 - s0) * SLICE;
-        const size_t first = slots.size();
-        for (int64_t sl = s0; sl < s1; ++sl) {
-            const int lanes = (int)std::min<int64_t>(SLICE, NI - sl * SLICE);
-            for (int j = 0; j < n; ++j)
-                for (int l = 0; l < lanes; ++l) {
-                    const int32_t c = col[(sl * n + j) * SLICE + l];
-                    if ((c < r0 || c >= r1) && place[c] < 0) {
-                        place[c] = 0;
-                        slots.push_back(c);
-                    }
-                }
-        }
-        std::sort(slots.begin() + first, slots.end());
-        const int64_t nh = (int64_t)(slots.size() - first);
-        if (rows + nh > 65535) return RBFFD_OK;
-        most = std::max(most, nh);
-        for (int64_t i = 0; i < nh; ++i) place[slots[first + i]] = (int32_t)(rows + i);
-        for (int64_t sl = s0; sl < s1; ++sl) {
-            const int lanes = (int)std::min<int64_t>(SLICE, NI - sl * SLICE);
-            for (int j = 0; j < n; ++j)
-                for (int l = 0; l < lanes; ++l) {
-                    const int64_t e = (sl * n + j) * SLICE + l;
-                    const int32_t c = col[e];
-                    lidx[e] = (uint16_t)(c >= r0 && c < r1 ? c - r0 : place[c]);
-                }
-        }
-        for (int64_t i = 0; i < nh; ++i) place[slots[first + i]] = -1;
-        off[b + 1] = (int32_t)slots.size();
-    }
-    if (slots.empty()) slots.push_back(0);
-    p->lk_bytes = sizeof(unsigned long long) *
-                  ((size_t)LINK_RING * 2 * NI + (size_t)LINK_RING * 2 * G + LINK_RING);
-    cudaError_t e = cudaMalloc((void**)&p->lk_idx, sizeof(uint16_t) * ent);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->lk_off, sizeof(int32_t) * off.size());
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->lk_slot, sizeof(int32_t) * slots.size());
-    if (e == cudaSuccess) e = cudaMalloc((void**)&p->lk_x, p->lk_bytes);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(p->lk_idx, lidx.data(), sizeof(uint16_t) * ent, cudaMemcpyHostToDevice,
-                            s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(p->lk_off, off.data(), sizeof(int32_t) * off.size(),
-                            cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(p->lk_slot, slots.data(), sizeof(int32_t) * slots.size(),
-                            cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    RBFFD_CHECK_CUDA(e);
+    const int64_t rows = (nsl + G - 1) / G * SLICE;
+    p->lk_max = 0;
+    for (int b = 0; b < G; ++b) p->lk_max = std::max<int64_t>(p->lk_max, listed[2 * b + 1]);
     p->lk_grid = G;
-    p->lk_max = most;
-    p->lk_ok = true;
+    p->lk_ok = p->lk_max <= LINK_CAP && rows + p->lk_max <= 65535;
     return RBFFD_OK;
+}
+
+// the linked kernel's launch: its dynamic shared memory, or false where it does
+// not fit
+static bool link_shape(const rbffd_plan* p, int mode, StepFn fn, int threads, unsigned* smem) {
+    int per_sm = 0;
+    *smem = link_smem(p->nslices, p->n, mode, p->lk_grid, p->lk_max);
+    if (!fn || allow_smem((const void*)fn, *smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn, threads, *smem) !=
+            cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        return false;
+    }
+    return true;
 }
 
 // halo slots of a block up to which the linked launch needs no rival (tune_shape)
@@ -1190,27 +1240,12 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
         (p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_RESIDENT)) && p->res_halo_set < -1) {
         int st0 = build_link(p, s);
         if (st0) return st0;
-        int dev = 0, optin = 0;
         for (int wide = 0; wide < 2 && p->lk_ok; ++wide) {
             TuneCand t;
             t.threads = wide ? RES_THREADS_WIDE : RES_THREADS_HOST;
             if (p->res_threads_set && t.threads != p->res_threads_set) continue;
             t.fn = pick_link(mode, p->n, t.threads);
-            if (!t.fn) continue;
-            t.smem = link_smem(p->nslices, p->n, mode, p->lk_grid, p->lk_max);
-            int per_sm = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess ||
-                cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-                    cudaSuccess ||
-                t.smem + 1024u > (unsigned)optin ||
-                allow_smem((const void*)t.fn, t.smem) != cudaSuccess ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)t.fn,
-                                                              t.threads, t.smem) !=
-                    cudaSuccess ||
-                per_sm < 1) {
-                cudaGetLastError();
-                continue;
-            }
+            if (!link_shape(p, mode, t.fn, t.threads, &t.smem)) continue;
             t.minb = 1;
             t.pdl = false;
             t.per_sm = 1;
@@ -2266,6 +2301,144 @@ static int power_stepwise(rbffd_plan* p, const StepArgs& A, const double* v0, in
     return RBFFD_OK;
 }
 
+// max over rows of sum_j |w_ij| into *out (IEEE bits)
+__global__ void row_abs_max(const double* __restrict__ w64, int64_t NI, int64_t nslices, int n,
+                            unsigned long long* out) {
+    unsigned long long m = 0;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t base = p / SLICE * (int64_t)n * SLICE + p % SLICE;
+        double a = 0.0;
+        for (int j = 0; j < n; ++j) a += fabs(w64[base + (int64_t)j * SLICE]);
+        m = max(m, abs_bits(a));
+    }
+    m = block_max_bits(m);
+    if (threadIdx.x == 0) red_max_relaxed(out, m);
+}
+
+// v <- 2^-e v with 2^e <= max < 2^(e+1) (bits in *mx; 0, subnormal or not finite: as it is)
+__global__ void scale_to_one(double* v, int64_t NI, const unsigned long long* mx) {
+    const unsigned ex = (unsigned)(*mx >> 52);
+    if (ex < 1u || ex > 2045u) return;
+    const double sc = bitsd((unsigned long long)(2046u - ex) << 52);
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
+         p += (int64_t)gridDim.x * blockDim.x)
+        v[p] = __dmul_rn(v[p], sc);
+}
+
+// partial sums of squares of y (s1) and of the ring's iterate x (s0)
+__global__ void link_norms(const double* __restrict__ y, const unsigned long long* __restrict__ x,
+                           int64_t NI, double* s0, double* s1) {
+    __shared__ double sh[2][256];
+    double a = 0.0, b = 0.0;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const double u = bitsd((x[2 * p] & 0xffffffffull) | (x[2 * p + 1] << 32));
+        a = __fma_rn(u, u, a);
+        b = __fma_rn(y[p], y[p], b);
+    }
+    sh[0][threadIdx.x] = a;
+    sh[1][threadIdx.x] = b;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if ((int)threadIdx.x < o)
+            for (int q = 0; q < 2; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        s0[blockIdx.x] = sh[0][0];
+        s1[blockIdx.x] = sh[1][0];
+    }
+}
+
+// The power iteration in the linked launch, for plans that may take it: y <- c W y
+// with c the power of two just below 1 / max row sum of |W|, so no component
+// grows, at most POWER_CHUNK iterations a launch, between which the vector is
+// scaled back (exactly).  *done false where the plan does not fit it or has
+// rows of no size.  200 iterations against the persistent launch: 10k rows, n = 12
+// 0.81 -> 0.48 ms; 90k, n = 30 2.06 -> 1.32, n = 24 2.96 -> 1.12.
+static constexpr int POWER_CHUNK = 64;
+
+static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int iters,
+                        double* rho, bool* done, cudaStream_t s) {
+    if (iters < 2 || !(p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_RESIDENT)))
+        return RBFFD_OK;
+    int st = build_link(p, s);
+    if (st) return st;
+    if (!p->lk_ok) return RBFFD_OK;
+    // a warp per slice where the block size allows it
+    const int threads = (p->nslices + p->lk_grid - 1) / p->lk_grid > RES_THREADS_HOST / 32 - 1 &&
+                                pick_link_power(p->n, RES_THREADS_WIDE)
+                            ? RES_THREADS_WIDE
+                            : RES_THREADS_HOST;
+    StepFn fn = pick_link_power(p->n, threads);
+    unsigned smem = 0;
+    if (!link_shape(p, MODE_SWEEP64, fn, threads, &smem)) return RBFFD_OK;
+    const int sms = device_sm_count();
+    constexpr int NP = 512;   // partial sums
+    double* part = p->scratch + 8;
+    unsigned long long* mx = reinterpret_cast<unsigned long long*>(p->scratch);   // [0] W, [1] v
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned long long), s));
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[0], 0, sizeof(double) * p->N, s));
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[1], 0, sizeof(double) * p->N, s));
+    gather_f<<<sms * 8, 256, 0, s>>>(v0, p->row_of_slot, p->NI, p->u[0]);
+    row_abs_max<<<sms * 4, 256, 0, s>>>(p->w64, p->NI, p->nslices, p->n, mx);
+    vec_max<<<sms, 256, 0, s>>>(p->u[0], p->NI, mx + 1);
+    norm_partials<<<NP, 256, 0, s>>>(p->u[0], p->NI, part + 2 * NP);
+    scale_to_one<<<sms, 256, 0, s>>>(p->u[0], p->NI, mx + 1);
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    unsigned long long wmax = 0;
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(&wmax, mx, sizeof(wmax), cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
+    const int ex = (int)(wmax >> 52);
+    if (ex < 2 || ex > 2040) return RBFFD_OK;   // nothing to scale by
+    const double sc = ldexp(1.0, 1023 - ex - 1);   // <= 1 / max row sum
+    int left = iters, cur = 0, last = 0;
+    while (left > 0) {
+        // the last launch has at least two iterations: its last two iterates are summed
+        const int k = left <= POWER_CHUNK ? left : left == POWER_CHUNK + 1 ? POWER_CHUNK - 1
+                                                                           : POWER_CHUNK;
+        if ((st = ctrl_reset(p, sc, 0.0, k, s))) return st;
+        StepArgs A = A0;
+        A.u0 = p->u[cur];
+        A.u1 = p->u[cur ^ 1];
+        RBFFD_CHECK_CUDA(link_args(p, k, &A, s));
+        StepCtrl* c = p->ctrl;
+        void* args[] = {(void*)&A, (void*)&c};
+        const cudaError_t e = cudaLaunchCooperativeKernel((const void*)fn, dim3(p->lk_grid),
+                                                          dim3(threads), args, smem, s);
+        if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+            cudaGetLastError();
+            return RBFFD_OK;
+        }
+        RBFFD_CHECK_CUDA(e);
+        left -= k;
+        cur ^= k & 1;
+        last = k;
+        if (left > 0) {
+            RBFFD_CHECK_CUDA(cudaMemsetAsync(mx + 1, 0, sizeof(unsigned long long), s));
+            vec_max<<<sms, 256, 0, s>>>(p->u[cur], p->NI, mx + 1);
+            scale_to_one<<<sms, 256, 0, s>>>(p->u[cur], p->NI, mx + 1);
+        }
+    }
+    // || y_K || / (sc || y_{K-1} ||): the result and the iterate before it in the ring
+    double* psc = part + 3 * NP;
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(psc, &sc, sizeof(sc), cudaMemcpyHostToDevice, s));
+    link_norms<<<NP, 256, 0, s>>>(p->u[cur], p->lk_x + (size_t)((last - 1) % LINK_RING) * 2 * p->NI,
+                                  p->NI, part, part + NP);
+    power_rho<<<1, 256, 0, s>>>(part + 2 * NP, NP, part, NP, part + NP, NP, psc, p->scratch);
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    int how = 0;
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(&how, &p->ctrl->done, sizeof(int), cudaMemcpyDeviceToHost,
+                                     s));
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(rho, p->scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
+    if (how == DONE_TIMEOUT) return done_status(how);
+    if (how != DONE_CAP) *rho = NAN;   // not finite on the way
+    *done = true;
+    return RBFFD_OK;
+}
+
 // the power iteration in one cooperative launch; *done false where the device
 // cannot hold the grid at once
 static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int iters,
@@ -2326,7 +2499,8 @@ extern "C" int rbffd_stable_dt(rbffd_plan* p, const double* v0, int iters, doubl
     double rho = 0.0;
     bool done = false;
     if (p->NN == 0) {   // (the Neumann update between iterations needs launches of its own)
-        int st = power_launch(p, A, v0, iters, &rho, &done, s);
+        int st = power_linked(p, A, v0, iters, &rho, &done, s);
+        if (!st && !done) st = power_launch(p, A, v0, iters, &rho, &done, s);
         if (st) return st;
     }
     if (!done) {

@@ -1,5 +1,6 @@
-"""The power iteration's single launch (plans without Neumann nodes) against the oracle's
-iteration: one, two and many iterations (the norms come from different kernels), stencil sizes
+"""The power iteration's launches (plans without Neumann nodes: one persistent launch, or linked
+ones of up to 64 iterations) against the oracle's iteration: one, two and many iterations, about
+a launch's 64 too (the norms come from different kernels), stencil sizes
 with and without a compiled kernel, node orders, int32 indices, one partial slice; vectors with
 no direction or with NaN are refused."""
 import numpy as np
@@ -29,15 +30,16 @@ def T(x):
 
 @pytest.mark.parametrize("d,Kg,m,n,flags", [(2, 60, 2, 12, 0), (2, 45, 4, 30, 64),
                                             (2, 45, 4, 31, 2), (2, 30, 4, 30, 32),
+                                            (2, 100, 2, 12, 64), (2, 160, 4, 31, 64),
                                             (2, 40, 6, 56, 0), (3, 12, 4, 70, 0),
-                                            (2, 4, 1, 6, 0)])
+                                            (3, 12, 4, 70, 64), (2, 4, 1, 6, 0)])
 def test_radius_equals_the_oracles(rb, orc, d, Kg, m, n, flags):
     p = build(orc, d, Kg, m, seed=17, n=n)
     plan = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w), flags, 3)
     v0 = gen.random_vector(p.NI, 5)
     # each iteration's sums of n + N terms round within (n + N) 2^-53 of the exact ones and
     # the radius is stationary to first order; the repository's bound is 1e-9
-    for iters in (1, 2, 3, 200):
+    for iters in (1, 2, 3, 63, 65, 200):
         rho = orc.power_rho(p.w, p.idx, p.interior, p.N, v0, iters)
         for scale in (1.0, 1e-100, 1e100):
             got = plan.stable_dt(T(v0 * scale), iters, 1.05)[1]
