@@ -416,6 +416,21 @@ RBFFD_API int rbffd_solve_explicit(rbffd_plan* plan, const double* f, double* u,
                          double* h_res_out, void* stream);
 
 /*
+ * rbffd_solve_record - K explicit steps (FP64, no stop tolerance) that keep
+ * iterates for rbffd_adjoint_w: as K / seg calls of rbffd_solve_explicit of seg
+ * steps each (the divergence test starts over with each), with u before each of
+ * them kept, in one call.
+ *   f, u, dt as for rbffd_solve_explicit.  ckpt [ckpt_rows][N] out, caller's
+ *   order (NULL: none kept), ckpt_rows >= ceil(K / seg).
+ *   h_every_out (host): the spacing of the kept iterates, u^0, u^every, ...: seg,
+ *   or 1 when ckpt_rows >= K and the plan can keep every iterate as it runs
+ *   (linked).  Returns as rbffd_solve_explicit, RBFFD_OK after K steps.
+ */
+RBFFD_API int rbffd_solve_record(rbffd_plan* plan, const double* f, double* u, double dt,
+                                 int64_t K, int64_t seg, double* ckpt, int64_t ckpt_rows,
+                                 int64_t* h_every_out, void* stream);
+
+/*
  * rbffd_plan_stats - what the last solve on this plan did (host outputs, may
  * be NULL): h_loop_ms, the GPU time of its step loops measured with CUDA
  * events recorded on the caller's stream around the step launches;

@@ -60,9 +60,10 @@ EXPORTED = [
     "rbffd_nodes_pds", "rbffd_nodes_pds_cap", "rbffd_weights_batch", "rbffd_transpose",
     "rbffd_plan_set_wait", "rbffd_fp64_fma_rate", "rbffd_plan_set_resident_halo",
     "rbffd_plan_set_block",
-    "rbffd_transpose_layout",
+    "rbffd_transpose_layout", "rbffd_solve_record",
 ]
 RBFFD_KNN_NOALLOC_MAX_NODES = 262144
+KEEP_ITERATES = 256 << 20   # bytes of iterates a differentiable solve may keep whole
 
 
 class RbffdError(RuntimeError):
@@ -100,6 +101,7 @@ def lib():
         "rbffd_plan_destroy": (I, [P]),
         "rbffd_plan_perm": (I, [P, P, P]),
         "rbffd_solve_explicit": (I, [P, P, P, D, I64, D, I, PI64, PD, P]),
+        "rbffd_solve_record": (I, [P, P, P, D, I64, I64, P, I64, PI64, P]),
         "rbffd_solve_dc": (I, [P, P, P, D, D, I64, I64, D, PI64, PI64, PD, P]),
         "rbffd_plan_set_dc": (I, [P, I64, D]),
         "rbffd_stable_dt": (I, [P, P, I, D, PD, PD, P]),
@@ -419,6 +421,21 @@ class Plan:
         _check(code, (RBFFD_OK, RBFFD_NOT_CONVERGED))
         return code, outer.value, inner.value, res.value
 
+    def solve_record(self, f, u, dt, K, seg, ckpt=None):
+        """K steps in place on ``u`` [N], keeping iterates in ``ckpt`` [rows, N] (rows >=
+        ceil(K / seg)).  Returns their spacing (seg, or 1 when the plan kept them all)."""
+        f = _dev(f, torch.float64, "f")
+        if not (u.is_cuda and u.dtype == torch.float64 and u.is_contiguous()):
+            raise ValueError("u must be a contiguous float64 CUDA tensor (updated in place)")
+        if ckpt is not None and not (ckpt.is_cuda and ckpt.dtype == torch.float64 and
+                                     ckpt.is_contiguous() and ckpt.shape[1] == self.N):
+            raise ValueError("ckpt must be a contiguous float64 CUDA tensor [rows, N]")
+        every = ctypes.c_int64(0)
+        _check(lib().rbffd_solve_record(self.handle, _ptr(f), _ptr(u), float(dt), int(K), int(seg),
+                                        _ptr(ckpt), 0 if ckpt is None else ckpt.shape[0],
+                                        ctypes.byref(every), _stream(self.device)))
+        return every.value
+
     def adjoint_w(self, f, ckpt, every, dLdu, K, dt):
         """Backward pass with the weight gradient from checkpoints ckpt [nseg, N] (caller
         order, u^0, u^every, ...) and dLdu = dL/du^K [N].
@@ -653,9 +670,10 @@ class ExplicitSolver:
 
     ``solver(f, g, w)`` returns u^K [N] from u^0 = 0 inside and g on the boundary
     (``g`` in the order of the boundary nodes, ascending).  Gradients flow to f, g
-    and (if it requires grad) the weights w [NI, n].  The forward keeps every
-    ``every``-th iterate (default ceil(sqrt(K))); the backward replays each
-    segment from its checkpoint to get the iterates the weight gradient needs."""
+    and (if it requires grad) the weights w [NI, n].  For the weight gradient the
+    forward keeps every ``every``-th iterate (default ceil(sqrt(K))), from which the
+    backward replays each segment, or, where they take no more than KEEP_ITERATES
+    bytes and the plan can keep them as it runs, all of them."""
 
     def __init__(self, xyz, is_bnd, interior, idx, K, dt, every=None, flags=0):
         self.xyz, self.is_bnd = xyz, is_bnd
@@ -689,14 +707,18 @@ class RBFFDExplicit(torch.autograd.Function):
         plan = solver.plan(w)
         u = torch.zeros(solver.N, dtype=torch.float64, device=f.device)
         u[solver.bnd] = g
-        ck = []
-        done = 0
-        while done < solver.K:
-            ck.append(u.clone())
-            steps = min(solver.every, solver.K - done)
-            plan.solve_explicit(f.contiguous(), u, solver.dt, steps, 0.0)
-            done += steps
-        ckpt = torch.stack(ck) if ck else u.clone()[None]
+        # without a weight gradient the backward needs no iterates; with one, all of them
+        # where they are small (nothing is replayed then), else every `every`-th
+        rows, every, ckpt = -(-solver.K // solver.every), solver.every, None
+        if ctx.needs_input_grad[2] and solver.K > 0:
+            if solver.K * solver.N * 8 <= KEEP_ITERATES:
+                rows = solver.K
+            ckpt = torch.empty((rows, solver.N), dtype=torch.float64, device=f.device)
+        if solver.K > 0:
+            every = plan.solve_record(f.contiguous(), u, solver.dt, solver.K, solver.every, ckpt)
+        if ckpt is None:
+            ckpt = u.clone()[None]
+        ctx.every = every
         ctx.solver = solver
         ctx.save_for_backward(f, ckpt)
         return u
@@ -709,7 +731,7 @@ class RBFFDExplicit(torch.autograd.Function):
         grad_u = grad_u.contiguous()
         gw = None
         if ctx.needs_input_grad[2]:
-            gw, gf, gg, _ = plan.adjoint_w(f.contiguous(), ckpt, solver.every, grad_u, solver.K,
+            gw, gf, gg, _ = plan.adjoint_w(f.contiguous(), ckpt, ctx.every, grad_u, solver.K,
                                            solver.dt)
         else:
             gf, gg, _ = plan.adjoint(grad_u, solver.K, solver.dt, want_lam0=False)

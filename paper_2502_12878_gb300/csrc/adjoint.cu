@@ -607,10 +607,14 @@ __global__ void wgrad_unpack(const double* __restrict__ G, const int32_t* row_of
     }
 }
 
-__global__ void ckpt_gather(const double* u, const int32_t* perm, int64_t N, double* out) {
+// `rows` checkpoints [rows][N] into slot order
+__global__ void ckpt_gather(const double* u, const int32_t* perm, int64_t N, int rows,
+                            double* out) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N;
-         p += (int64_t)gridDim.x * blockDim.x)
-        out[p] = u[perm[p]];
+         p += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t q = perm[p];
+        for (int r = 0; r < rows; ++r) out[r * N + p] = u[r * N + q];
+    }
 }
 
 // reverse-step shapes the tuner times: (phase width, register budget), each
@@ -922,7 +926,11 @@ extern "C" int rbffd_adjoint_w(rbffd_plan* p, const double* f, const double* ckp
     const unsigned G = (unsigned)sms * 8;
     const int64_t N = p->N, NI = p->NI;
     const int n = p->n;
-    const int64_t seg = std::min<int64_t>(every, std::max<int64_t>(K, 1));
+    // steps between replays; with every iterate kept nothing is replayed, and a
+    // group of steps is taken at a time
+    const bool all = every == 1;
+    const int64_t span = all ? WG_STEPS : every;
+    const int64_t seg = std::min<int64_t>(span, std::max<int64_t>(K, 1));
     // the segment's iterates, the lambdas of up to WG_STEPS steps and the one after
     // them (a ring), the weight gradient's accumulator
     constexpr int RING = WG_STEPS + 1;
@@ -978,16 +986,18 @@ extern "C" int rbffd_adjoint_w(rbffd_plan* p, const double* f, const double* ckp
         RBFFD_REPLAY(71)
     }
 #undef RBFFD_REPLAY
-    const int64_t nseg = (K + every - 1) / every;
+    const int64_t nseg = (K + span - 1) / span;
     const unsigned wgrid =
         (unsigned)std::max<int64_t>(1, std::min<int64_t>((NI + 255) / 256, (int64_t)sms * 24));
     int cur = 0;   // lambda^{k+1} lives in lam(cur)
     bool first = true;
     for (int64_t sidx = nseg - 1; sidx >= 0; --sidx) {
-        const int64_t k0 = sidx * every, k1 = std::min(K, k0 + every);
-        // u^{k0} from its checkpoint, then replay u^{k0+1} .. u^{k1-1}
-        ckpt_gather<<<G, 256, 0, s>>>(ckpt + sidx * N, p->perm, N, U);
-        for (int64_t k = k0; k + 1 < k1; ++k)
+        const int64_t k0 = sidx * span, k1 = std::min(K, k0 + span);
+        // u^{k0} from its checkpoint, then replay u^{k0+1} .. u^{k1-1} (or all
+        // of them from theirs)
+        ckpt_gather<<<G, 256, 0, s>>>(ckpt + (all ? k0 : sidx) * N, p->perm, N,
+                                      all ? (int)(k1 - k0) : 1, U);
+        for (int64_t k = k0; !all && k + 1 < k1; ++k)
             RBFFD_CHECK_CUDA(launch_dependent(replay, rgrid, STEP_THREADS, s, A,
                                               (const double*)(U + (k - k0) * N),
                                               U + (k - k0 + 1) * N, dt));

@@ -204,6 +204,13 @@ struct StepArgs {
     unsigned long long* lk_res;   // [LINK_RING][blocks] two-word entries
     unsigned long long* lk_dec;   // [LINK_RING]
     unsigned lk_epoch;
+    // a recorded run (FP64): u^k for every k a multiple of rec_every, in the
+    // caller's node order, to rec [..][N] (NULL: none); and the divergence test
+    // starts over every lk_seg steps (0: never)
+    double* rec;
+    const int32_t* perm;
+    int rec_every;
+    long long lk_seg;
 };
 
 // iterates in the linked launch's ring, and how many steps a block may be ahead

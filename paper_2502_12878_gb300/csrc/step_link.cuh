@@ -121,8 +121,10 @@ __device__ __forceinline__ int link_decide(const StepArgs& A, StepCtrl* c, long 
     }
     if (!__all_sync(0xffffffffu, all)) return -1;
     const double R = bitsd(link_warp_max(m));
-    if (q == k0) *R0 = R;
-    const int dn = stop_rule(R, *R0, q, kmax, tol);
+    const long long in_seg = A.lk_seg > 0 ? (q - k0) % A.lk_seg : q - k0;
+    if (in_seg == 0) *R0 = R;
+    int dn = stop_rule(R, *R0, in_seg, kmax, tol);
+    if (dn == DONE_RUNNING && q + 1 >= kmax) dn = DONE_CAP;
     if (lane == 0) {
         st_relaxed(A.lk_dec + q % LINK_RING,
                    (unsigned long long)dn | ((unsigned long long)tag << 32));
@@ -389,6 +391,12 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
         unsigned long long* xn = X + rn * ring;
         B m = 0;
         bool bad = false, have = k == k0;   // the start iterate's halo is there
+        if constexpr (MODE == MODE_SWEEP64) {
+            if (A.rec && (k - k0) % A.rec_every == 0) {
+                double* to = A.rec + (k - k0) / A.rec_every * A.N;
+                for (int i = threadIdx.x; i < nown; i += TC) to[A.perm[r0 + i]] = vc[i];
+            }
+        }
         if (npoll > 0 && polls && !have) {
             for (int i = pstart; i < nint; i += pstep)
                 bad = !link_wait(xc, slot_s[i], tag, vc + rows + i, spin) || bad;

@@ -313,6 +313,32 @@ __global__ void scatter_u(const double* us, const int32_t* perm, int64_t NI, dou
         u[perm[p]] = us[p];
 }
 
+// the result of a run: u^k, k and so its buffer as the control block has it
+__global__ void scatter_result(const StepCtrl* c, const double* u0, const double* u1,
+                               const int32_t* perm, int64_t NI, double* u) {
+    const double* us = (c->k & 1) ? u1 : u0;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
+         p += (int64_t)gridDim.x * blockDim.x)
+        u[perm[p]] = us[p];
+}
+
+// an iterate in slot order to the caller's order, boundary slots too; the
+// boundary's values alone to `rows` records
+__global__ void record_iterate(const double* us, const int32_t* perm, int64_t N, double* out) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < N;
+         p += (int64_t)gridDim.x * blockDim.x)
+        out[perm[p]] = us[p];
+}
+__global__ void record_boundary(const double* us, const int32_t* perm, int64_t NI, int64_t N,
+                                int64_t rows, double* out) {
+    const int64_t nb = N - NI;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nb * rows;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = NI + i % nb;
+        out[i / nb * N + perm[p]] = us[p];
+    }
+}
+
 // ---------------------------------------------------- Neumann boundary nodes
 // Before each step, every Neumann node b takes the value that meets its
 // normal-derivative condition with the previous iterate of its other support
@@ -771,6 +797,10 @@ static StepArgs make_args(const rbffd_plan* p) {
     A.lk_max = 0;
     A.lk_x = A.lk_res = A.lk_dec = nullptr;
     A.lk_epoch = 0;
+    A.rec = nullptr;
+    A.perm = p->perm;
+    A.rec_every = 1;
+    A.lk_seg = 0;
     return A;
 }
 
@@ -860,6 +890,8 @@ static int persistent_grid(StepFn fn, const rbffd_plan* p) {
 // reset the control block for a run of at most max_steps steps; `held`:
 // arrivals the persistent barrier waits for beyond the grid's (0 but in a
 // test of the timeout path, rbffd_plan_set_wait)
+__global__ void ctrl_set(StepCtrl* c, const StepCtrl v) { *c = v; }
+
 static int ctrl_reset(rbffd_plan* p, double dt, double tol, long long max_steps, cudaStream_t s,
                       int held = 0) {
     StepCtrl h;
@@ -870,7 +902,8 @@ static int ctrl_reset(rbffd_plan* p, double dt, double tol, long long max_steps,
     h.done = max_steps <= 0 ? DONE_CAP : DONE_RUNNING;
     h.held = held;
     h.spin_limit = p->spin_limit;
-    RBFFD_CHECK_CUDA(cudaMemcpyAsync(p->ctrl, &h, sizeof(h), cudaMemcpyHostToDevice, s));
+    ctrl_set<<<1, 1, 0, s>>>(p->ctrl, h);
+    RBFFD_CHECK_CUDA(cudaGetLastError());
     return RBFFD_OK;
 }
 
@@ -1583,8 +1616,16 @@ static int prepare_mode(rbffd_plan* p, int mode, double dt, double tol, long lon
 
 // run the step loop of `mode` until the control block says done.
 // Reads back done / k / res_last.
+// `u_out`: the caller's array for the result (FP64 sweep), written behind the
+// steps so that one wait covers both; `rec`: a recorded run (linked launch only).
+struct RecordTo {
+    double* rec;
+    int every;
+    long long seg;
+};
 static int run_steps(rbffd_plan* p, int mode, double dt, double tol, long long max_steps,
-                     cudaStream_t s, long long* steps, double* res, int* done) {
+                     cudaStream_t s, long long* steps, double* res, int* done,
+                     double* u_out = nullptr, const RecordTo* rec = nullptr) {
     int st = ctrl_reset(p, dt, tol, max_steps, s, p->held_arrivals);
     if (st) return st;
     StepCtrl h;
@@ -1610,6 +1651,11 @@ static int run_steps(rbffd_plan* p, int mode, double dt, double tol, long long m
             A.halo = p->resident[mi] ? p->res_halo[mi] : 0;
             far_args(p, mi, &A);
             if (p->link[mi]) RBFFD_CHECK_CUDA(link_args(p, max_steps, &A, s));
+            if (rec) {
+                A.rec = rec->rec;
+                A.rec_every = rec->every;
+                A.lk_seg = rec->seg;
+            }
             StepCtrl* c = p->ctrl;
             void* args[] = {(void*)&A, (void*)&c};
             RBFFD_CHECK_CUDA(cudaEventRecord((cudaEvent_t)p->ev[0], s));
@@ -1654,6 +1700,12 @@ static int run_steps(rbffd_plan* p, int mode, double dt, double tol, long long m
             RBFFD_CHECK_CUDA(cudaGetLastError());
             p->last_launches += launched + 1;
         }
+    }
+    if (u_out) {
+        scatter_result<<<device_sm_count() * 8, 256, 0, s>>>(p->ctrl, p->u[0], p->u[1], p->perm,
+                                                             p->NI, u_out);
+        RBFFD_CHECK_CUDA(cudaGetLastError());
+        p->last_launches += 1;
     }
     RBFFD_CHECK_CUDA(cudaMemcpyAsync(&h, p->ctrl, sizeof(h), cudaMemcpyDeviceToHost, s));
     RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
@@ -2241,17 +2293,15 @@ extern "C" int rbffd_solve_explicit(rbffd_plan* p, const double* f, double* u, d
     long long steps = 0;
     double R = 0.0;
     int done = 0;
-    st = run_steps(p, MODE_SWEEP64, dt, tol, max_steps, s, &steps, &R, &done);
+    st = run_steps(p, MODE_SWEEP64, dt, tol, max_steps, s, &steps, &R, &done, u);
     if (st) return st;
-    int sms = device_sm_count();
-    scatter_u<<<sms * 8, 256, 0, s>>>(p->u[steps & 1], p->perm, p->NI, u);
-    p->last_launches += 1;
     if (p->NN > 0) {
-        neumann_out<<<sms * 2, 256, 0, s>>>(p->nslot, p->u[steps & 1], p->perm, p->NN, u);
+        neumann_out<<<device_sm_count() * 2, 256, 0, s>>>(p->nslot, p->u[steps & 1], p->perm,
+                                                          p->NN, u);
         p->last_launches += 1;
+        RBFFD_CHECK_CUDA(cudaGetLastError());
+        RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
     }
-    RBFFD_CHECK_CUDA(cudaGetLastError());
-    RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
     if (h_steps_out) *h_steps_out = steps;
     if (h_res_out) *h_res_out = R;
     if (max_steps == 0) return RBFFD_NOT_CONVERGED;
@@ -2487,6 +2537,64 @@ static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int 
     RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
     if (stopped == DONE_TIMEOUT) return done_status(DONE_TIMEOUT);
     *done = true;
+    return RBFFD_OK;
+}
+
+extern "C" int rbffd_solve_record(rbffd_plan* p, const double* f, double* u, double dt, int64_t K,
+                                  int64_t seg, double* ckpt, int64_t ckpt_rows,
+                                  int64_t* h_every_out, void* stream) {
+    clear_error();
+    RBFFD_ARG(p && f && u && h_every_out, "rbffd_solve_record: NULL argument");
+    RBFFD_ARG(dt > 0.0 && isfinite(dt), "rbffd_solve_record: dt must be positive and finite");
+    RBFFD_ARG(K >= 0 && seg >= 1 && (!ckpt || ckpt_rows >= (K + seg - 1) / seg),
+              "rbffd_solve_record: bad K / seg / ckpt_rows");
+    *h_every_out = seg;
+    cudaStream_t s = as_stream(stream);
+    int st = load_problem(p, f, u, s);
+    if (st) return st;
+    const int sms = device_sm_count();
+    if (K == 0) return RBFFD_OK;
+    if ((st = ctrl_reset(p, dt, 0.0, K, s, p->held_arrivals))) return st;
+    if ((st = prepare_mode(p, MODE_SWEEP64, dt, 0.0, K, s))) return st;
+    long long steps = 0;
+    double R = 0.0;
+    int done = 0;
+    if (p->persist[0] && p->link[0]) {
+        // one run, recorded by the launch itself: every step where that fits
+        RecordTo rec;
+        rec.rec = ckpt;
+        rec.every = ckpt_rows >= K ? 1 : (int)std::min<int64_t>(seg, 0x7fffffff);
+        rec.seg = seg;
+        if (ckpt) {
+            *h_every_out = rec.every;
+            record_boundary<<<sms * 4, 256, 0, s>>>(p->u[0], p->perm, p->NI, p->N,
+                                                    (K + rec.every - 1) / rec.every, ckpt);
+            RBFFD_CHECK_CUDA(cudaGetLastError());
+            p->last_launches += 1;
+        }
+        st = run_steps(p, MODE_SWEEP64, dt, 0.0, K, s, &steps, &R, &done, u, &rec);
+        if (st) return st;
+        return done == DONE_CAP ? RBFFD_OK : done_status(done);
+    }
+    for (int64_t k = 0; k < K; k += seg) {
+        if (ckpt)
+            record_iterate<<<sms * 8, 256, 0, s>>>(p->u[0], p->perm, p->N,
+                                                   ckpt + k / seg * p->N);
+        RBFFD_CHECK_CUDA(cudaGetLastError());
+        const int64_t m = std::min(seg, K - k);
+        st = run_steps(p, MODE_SWEEP64, dt, 0.0, m, s, &steps, &R, &done,
+                       k + m == K ? u : nullptr);
+        if (st) return st;
+        if (done != DONE_CAP) {
+            scatter_u<<<sms * 8, 256, 0, s>>>(p->u[steps & 1], p->perm, p->NI, u);
+            cudaStreamSynchronize(s);
+            return done_status(done);
+        }
+        // a run starts from u[0], and its boundary (and Neumann) slots are in both
+        if (k + m < K && (m & 1))
+            RBFFD_CHECK_CUDA(cudaMemcpyAsync(p->u[0], p->u[1], sizeof(double) * p->N,
+                                             cudaMemcpyDeviceToDevice, s));
+    }
     return RBFFD_OK;
 }
 
