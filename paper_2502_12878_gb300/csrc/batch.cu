@@ -12,10 +12,11 @@
 // non-finite, divergence).  One-block teams synchronise with __syncthreads
 // and gather the iterate through L1 (their own writes are visible after the
 // barrier); larger teams use a per-domain barrier whose waits give up after
-// ~2 s (RBFFD_ERR_TIMEOUT) and gather through L2 (.cg), because other blocks
-// of the same launch rewrite the iterate.  Slices read the plan's 16-bit
-// neighbour codes where it has them, and each warp prefetches its next
-// slice's planes into L2 (bulk prefetch) before it sweeps the current one.
+// ~2 s (RBFFD_ERR_TIMEOUT), because other blocks of the same launch rewrite
+// the iterate; how they gather depends on the register budget (batch_kernel).
+// Slices read the plan's 16-bit neighbour codes where it has them, and a warp
+// may prefetch its next slice's planes into L2 (bulk prefetch) before it
+// sweeps the current one.
 //
 // The per-call inputs (the caller's f / u pointers, dt, tol, step caps) are
 // copied into a device table at a fixed address, so one captured graph -
@@ -199,8 +200,9 @@ __device__ __forceinline__ void bprefetch(const DomDesc& D, int64_t sl) {
                      "r"(plane * 4u) : "memory");
 }
 
-// one step of domain D over the slices of this team member; returns max |r| bits
-template <int NN, bool COH, int CH>
+// one step of domain D over the slices of this team member; returns max |r|
+// bits.  PF: prefetch the warp's next slice first.
+template <int NN, bool COH, bool PF, int CH>
 __device__ __noinline__ unsigned long long bstep(const DomDesc& D, int par, double dt, int64_t s0,
                                                  int64_t stride) {
     const int lane = threadIdx.x & 31;
@@ -211,7 +213,7 @@ __device__ __noinline__ unsigned long long bstep(const DomDesc& D, int par, doub
         const int64_t row = sl * SLICE + lane;
         const int64_t base = sl * (int64_t)D.n * SLICE + lane;
         const int4 sb = D.col16 ? __ldg(D.sbase + sl) : make_int4(-1, -1, -1, -1);
-        if (lane == 0) bprefetch(D, sl + stride);
+        if (PF && lane == 0) bprefetch(D, sl + stride);
         if (row < D.NI) {
             const double fi = bld_cs(D.fs + row);
             const double ui = COH ? bld_cg(uin + row) : bld_ca(uin + row);
@@ -226,14 +228,14 @@ __device__ __noinline__ unsigned long long bstep(const DomDesc& D, int par, doub
     return m;
 }
 
-template <bool COH, int CH>
+template <bool COH, bool TIGHT, int CH>
 __device__ unsigned long long bstep_any(const DomDesc& D, int par, double dt, int64_t s0,
                                         int64_t stride) {
     switch (D.n) {
-        case 12: return bstep<12, COH, CH>(D, par, dt, s0, stride);
-        case 30: return bstep<30, COH, CH>(D, par, dt, s0, stride);
-        case 56: return bstep<56, COH, CH>(D, par, dt, s0, stride);
-        default: return bstep<0, COH, CH>(D, par, dt, s0, stride);
+        case 12: return bstep<12, COH, true, CH>(D, par, dt, s0, stride);
+        case 30: return bstep<30, COH, !TIGHT, CH>(D, par, dt, s0, stride);
+        case 56: return bstep<56, COH, !TIGHT, CH>(D, par, dt, s0, stride);
+        default: return bstep<0, COH, true, CH>(D, par, dt, s0, stride);
     }
 }
 
@@ -277,8 +279,7 @@ __device__ __forceinline__ int bdecide(DomState* st, const DomCall& C, int rank,
 }
 
 // one domain's solve by one team member (rank of size blocks); returns false
-// when a team wait gave up.  CH: neighbours per load phase (8 where the
-// register budget is below 80 per thread).  A one-block team decides right
+// when a team wait gave up.  A one-block team decides right
 // after each step (its residual is the block's).  Larger teams end a step
 // with a counter barrier (each block adds its max |r| to the step's residual
 // slot and its arrival to the domain's counter - both fire-and-forget, the
@@ -287,7 +288,7 @@ __device__ __forceinline__ int bdecide(DomState* st, const DomCall& C, int rank,
 // step: the same rule to the same value in every member, so the team stops
 // together.  A stop wastes that next step, which writes the other buffer; the
 // result u^{k+1} is untouched.  Rank 0 clears the slot step k + 2 will use.
-template <int CH>
+template <bool TIGHT, int CH>
 __device__ bool run_domain(const TeamDesc T, const DomDesc* __restrict__ desc,
                            const DomCall* __restrict__ call, DomState* state,
                            unsigned long long* wmax, int* s_stop) {
@@ -304,8 +305,9 @@ __device__ bool run_domain(const TeamDesc T, const DomDesc* __restrict__ desc,
     if (threadIdx.x == 0 && T.rank == 0) st->t_start = gtimer();
     for (long long k = 0; k < C.max_steps; ++k) {
         unsigned long long m = T.size == 1
-                                   ? bstep_any<false, CH>(D, (int)(k & 1), C.dt, s0, stride)
-                                   : bstep_any<true, CH>(D, (int)(k & 1), C.dt, s0, stride);
+                                   ? bstep_any<false, TIGHT, CH>(D, (int)(k & 1), C.dt, s0, stride)
+                                   : bstep_any<!TIGHT, TIGHT, CH>(D, (int)(k & 1), C.dt, s0,
+                                                                  stride);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (lane == 0) wmax[wid] = m;
@@ -357,16 +359,32 @@ __device__ bool run_domain(const TeamDesc T, const DomDesc* __restrict__ desc,
     return true;
 }
 
+// Bound by load latency: a step's planes come from L2 and a row's 12..56
+// gathers hit lines its neighbours have just brought in.  With 64 registers a
+// thread (1024 threads an SM, TIGHT) a row's loads go out in phases of 20
+// neighbours, teams of several blocks gather through L1 as well (weak loads:
+// the team barrier's acquire by thread 0 and the block barrier after it order
+// them behind the other blocks' writes, and a step writes only the other
+// buffer), and the wide stencils leave out the prefetch - 32 warps hide the
+// plane's latency and the prefetch's L2 requests only compete.  20 domains of
+// 5k..100k nodes, n = 12, 30 and 56, 200 steps, kernel time: 1024-thread
+// blocks 11.66 -> 10.39 ms (phases of 8 before; L1 alone 11.40, and without
+// the prefetch 10.76; phases of 16: 10.53, with .cg 10.86, with the prefetch
+// 11.32; of 24, 28, 56: 10.82, 10.94, 13.0), two blocks of 512 10.98 -> 9.92.
+// With more registers and so fewer warps the prefetch and .cg stay: L1 takes
+// 512-thread blocks with 128 registers from 12.5 to 13.3 ms, without the
+// prefetch to 15.4.
 template <int MINB, int TH>
 __global__ void __launch_bounds__(TH, MINB)
     batch_kernel(const DomDesc* __restrict__ desc, const DomCall* __restrict__ call,
                  DomState* state, const TeamDesc* __restrict__ assign,
                  const int* __restrict__ first) {
-    constexpr int CH = 65536 / (TH * MINB) >= 80 ? 16 : 8;
+    constexpr bool TIGHT = 65536 / (TH * MINB) < 80;
+    constexpr int CH = TIGHT ? 20 : 16;
     __shared__ unsigned long long wmax[BATCH_MAX_WARPS];
     __shared__ int s_stop;
     for (int a = first[blockIdx.x]; a < first[blockIdx.x + 1]; ++a)
-        if (!run_domain<CH>(assign[a], desc, call, state, wmax, &s_stop)) return;
+        if (!run_domain<TIGHT, CH>(assign[a], desc, call, state, wmax, &s_stop)) return;
 }
 
 // gather f and u of every domain into its plan (one launch for all domains)
