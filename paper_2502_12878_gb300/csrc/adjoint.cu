@@ -279,9 +279,8 @@ __global__ void scan64_single(const int64_t* in, int64_t n, int64_t* out) {
 }
 
 // Ordered streaming loads: asm volatile keeps the loads of one phase ahead of
-// the first use, so each thread has 2*CH loads and then CH gathers in flight
-// (plain loads were issued one dependent pair at a time).  CH = 8 with four
-// 256-thread blocks per SM fits 64 registers without spills.
+// the first use, so each thread has 2*M loads and then M gathers in flight
+// (plain loads were issued one dependent pair at a time).
 __device__ __forceinline__ double adj_ld_cs(const double* p) {
     double v;
     asm volatile("ld.global.cs.f64 %0, [%1];" : "=d"(v) : "l"(p));
@@ -311,51 +310,69 @@ __device__ __forceinline__ int32_t adj_decode16(uint32_t v, const int4& b) {
     return base + (int32_t)(v & 0x3fffu);
 }
 
-// sum over a column's L stored entries (stride SLICE) of w * lam[row], an fma
-// chain from 0 in entry order; loads in phases of CH (rows, weights, then
-// the gathers).  I16: rows as 16-bit codes against the slice's bases.
-// sum over a column's L stored entries (stride SLICE) of w * lam[row], an fma
-// chain from 0 in entry order; loads in phases of CH (rows, weights, then
-// the gathers).  I16: each entry's 16-bit code is decoded against the
-// slice's window bases, or, in a slice the windows cannot cover (sb.x < 0),
-// is the entry's own position in the slice, which reads its int32 row.
+// M entries of a column (stride SLICE): rows, weights, then the gathers, then
+// the fma chain.  I16: each entry's 16-bit code is decoded against the slice's
+// window bases, or, in a slice the windows cannot cover (sb.x < 0), is the
+// entry's own position in the slice, which reads its int32 row.
+template <int M, bool I16>
+__device__ __forceinline__ void adj_phase(const double* wp, const void* rp, const int32_t* rows,
+                                          const int4& sb, const double* __restrict__ lam,
+                                          double& acc) {
+    int32_t r[M];
+    double wv[M], lv[M];
+#pragma unroll
+    for (int t = 0; t < M; ++t) {
+        if constexpr (I16)
+            r[t] = (int32_t)adj_ld_cs((const uint16_t*)rp + t * SLICE);
+        else
+            r[t] = adj_ld_cs((const int32_t*)rp + t * SLICE);
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t) wv[t] = adj_ld_cs(wp + t * SLICE);
+    if constexpr (I16) {
+        if (sb.x >= 0) {
+#pragma unroll
+            for (int t = 0; t < M; ++t) r[t] = adj_decode16((uint32_t)r[t], sb);
+        } else {
+#pragma unroll
+            for (int t = 0; t < M; ++t) r[t] = adj_ld_cs(rows + r[t]);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t) lv[t] = adj_ld_nc(lam + r[t]);
+#pragma unroll
+    for (int t = 0; t < M; ++t) acc = __fma_rn(wv[t], lv[t], acc);
+}
+
+// the last rem <= M entries as one phase of exactly that many
+template <int M, bool I16>
+__device__ __forceinline__ void adj_rest(const double* wp, const void* rp, const int32_t* rows,
+                                         const int4& sb, const double* __restrict__ lam, int rem,
+                                         double& acc) {
+    if constexpr (M > 0) {
+        if (rem == M) adj_phase<M, I16>(wp, rp, rows, sb, lam, acc);
+        else adj_rest<M - 1, I16>(wp, rp, rows, sb, lam, rem, acc);
+    }
+}
+
+// sum over a column's L stored entries of w * lam[row], an fma chain from 0 in
+// entry order, in phases of CH and one shorter one.  L is the same for the
+// whole warp, so the length of the last phase is a branch and no load carries
+// a predicate: with phases of CH under `j < L` the predicates outlived the
+// ordered loads and were spilled (184 bytes a thread at CH = 8 and 64
+// registers, 2.1 million local requests a step at 998k columns).
 template <int CH, bool I16>
 __device__ __forceinline__ double adj_col_sum(const double* wp, const void* rp,
                                               const int32_t* rows, const int4& sb,
                                               const double* __restrict__ lam, int L) {
     double acc = 0.0;
-    for (int j0 = 0; j0 < L; j0 += CH) {
-        int32_t r[CH];
-        double wv[CH], lv[CH];
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < L) {
-                if constexpr (I16)
-                    r[t] = (int32_t)adj_ld_cs((const uint16_t*)rp + (int64_t)(j0 + t) * SLICE);
-                else
-                    r[t] = adj_ld_cs((const int32_t*)rp + (int64_t)(j0 + t) * SLICE);
-            }
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < L) wv[t] = adj_ld_cs(wp + (int64_t)(j0 + t) * SLICE);
-        if constexpr (I16) {
-            if (sb.x >= 0) {
-#pragma unroll
-                for (int t = 0; t < CH; ++t)
-                    if (j0 + t < L) r[t] = adj_decode16((uint32_t)r[t], sb);
-            } else {
-#pragma unroll
-                for (int t = 0; t < CH; ++t)
-                    if (j0 + t < L) r[t] = adj_ld_cs(rows + r[t]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < L) lv[t] = adj_ld_nc(lam + r[t]);
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < L) acc = __fma_rn(wv[t], lv[t], acc);
+    int j0 = 0;
+    for (; j0 + CH <= L; j0 += CH) {
+        adj_phase<CH, I16>(wp, rp, rows, sb, lam, acc);
+        wp += CH * SLICE;
+        rp = (const char*)rp + CH * SLICE * (I16 ? 2 : 4);
     }
+    adj_rest<CH - 1, I16>(wp, rp, rows, sb, lam, L - j0, acc);
     return acc;
 }
 
@@ -365,35 +382,24 @@ __device__ __forceinline__ double adj_col_sum(const double* wp, const void* rp,
 // (padding entries carry weight 0, so they add exact zeros).  Shapes: CH
 // entries per load phase (rows, weights, then gathers) and a register budget
 // for MINB resident blocks of 256 threads; every shape, and either row form,
-// gives the same bits.  One lane prefetches the warp's next slice (weight
-// plane and row codes, or rows when the plan keeps int32 indices) into L2:
-// both planes start on 16-byte boundaries (slice offsets are multiples of 32
-// entries) and span a multiple of 16 bytes.
+// gives the same bits.  Bound by the latency of the entry loads with the FP64
+// pipe and HBM both near 50 us a step at 998k columns of 30: 73.9 -> 62.9 us
+// a step there, n = 12 38.3 -> 31.5, 89k columns 11.6 -> 9.8, 10k of 12 4.09
+// -> 3.29, n = 56 at 250k 38.4 -> 33.2, 3D n = 70 40.9 -> 35.1, from phases
+// without predicates and from leaving out a bulk prefetch of the warp's next
+// slice (65.7 us with it: with 32 warps or more in flight it only competes).
 template <int CH, bool I16>
 __device__ __forceinline__ void adj_slices(const Transpose& T, const int64_t NI, const double dt,
                                            const double* __restrict__ lam,
                                            double* __restrict__ lam_out,
                                            double* __restrict__ S) {
     const int lane = threadIdx.x & 31;
-    const int64_t nsl_int = (NI + SLICE - 1) / SLICE;
-    const int64_t stride = (int64_t)gridDim.x * (blockDim.x / 32);
-    for (int64_t s = (int64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); s < nsl_int;
+    // (columns are int32 indices, so slices and their counters are too)
+    const int nsl_int = (int)((NI + SLICE - 1) / SLICE);
+    const int stride = (int)(gridDim.x * (blockDim.x / 32));
+    for (int s = (int)(blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)); s < nsl_int;
          s += stride) {
-        if (lane == 0 && s + stride < nsl_int) {
-            const int64_t o = __ldg(T.off + s + stride);
-            const unsigned Ln = (unsigned)__ldg(T.len + s + stride) * SLICE;
-            if (Ln) {
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(T.w + o),
-                             "r"(Ln * 8u) : "memory");
-                if (I16)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(T.row16 + o),
-                                 "r"(Ln * 2u) : "memory");
-                else
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(T.row + o),
-                                 "r"(Ln * 4u) : "memory");
-            }
-        }
-        const int64_t c = s * SLICE + lane;
+        const int64_t c = (int64_t)s * SLICE + lane;
         if (c >= NI) continue;
         const int L = __ldg(T.len + s);
         const int64_t off = __ldg(T.off + s);
@@ -620,11 +626,13 @@ __global__ void ckpt_gather(const double* u, const int32_t* perm, int64_t N, int
 // reverse-step shapes the tuner times: (phase width, register budget), each
 // with one warp per slice (the full grid) or a grid-stride loop over slices
 // on the resident blocks
-// (with 16-bit row codes the window bases need registers: at four blocks
-// per SM phases of 8 spill and phases of 6 or 7 fit)
-static const AdjStepFn adj_shapes[] = {adjoint_step<8, 4>,  adjoint_step<7, 4>,
-                                       adjoint_step<6, 4>,  adjoint_step<12, 3>,
-                                       adjoint_step<16, 2>, adjoint_step<8, 3>};
+// (998k columns of 30: 12 entries at 4 blocks and 8 at 5 win, 62.6-62.9 us,
+// 10 at 4 65.0, 8 at 4 65.8; 3D columns of 70: 16 at 3 35.1, 12 at 3 35.8, 12
+// at 4 36.8; 10k columns of 12: 16 at 3 3.30, 8 at 4 3.46; 16 at 2, 16 at 4
+// and 6 at 6 win nowhere)
+static const AdjStepFn adj_shapes[] = {adjoint_step<8, 4>,  adjoint_step<10, 4>,
+                                       adjoint_step<12, 4>, adjoint_step<8, 5>,
+                                       adjoint_step<12, 3>, adjoint_step<16, 3>};
 static constexpr int N_ADJ_SHAPES = 6;
 
 // one reverse step; `pdl`: as a programmatic dependent launch
