@@ -138,41 +138,71 @@ __device__ __forceinline__ int32_t bdecode16(uint32_t v, const int4& b) {
     return base + (int32_t)(v & 0x3fffu);
 }
 
-// sum_j w_j u[col_j], an fma chain from 0 in j order; loads in phases of CH
-// (indices, weights, then the gathers).  I16: 16-bit codes against the
-// slice's window bases `sb` (the same columns, fewer bytes).
+// M neighbours of a row, continuing the fma chain acc: indices, weights, then
+// the gathers.  I16: 16-bit codes against the slice's window bases `sb` (the
+// same columns, fewer bytes).
+template <int M, bool COH, bool I16>
+__device__ __forceinline__ double brow_phase(const double* __restrict__ w,
+                                             const void* __restrict__ colp, const int4& sb,
+                                             const double* __restrict__ u, double acc) {
+    int32_t c[M];
+    double wv[M], uv[M];
+#pragma unroll
+    for (int t = 0; t < M; ++t) {
+        if constexpr (I16) c[t] = (int32_t)bld_cs((const uint16_t*)colp + t * SLICE);
+        else c[t] = bld_cs((const int32_t*)colp + t * SLICE);
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t) wv[t] = bld_cs(w + t * SLICE);
+    if constexpr (I16) {
+#pragma unroll
+        for (int t = 0; t < M; ++t) c[t] = bdecode16((uint32_t)c[t], sb);
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t) uv[t] = COH ? bld_cg(u + c[t]) : bld_ca(u + c[t]);
+#pragma unroll
+    for (int t = 0; t < M; ++t) acc = __fma_rn(wv[t], uv[t], acc);
+    return acc;
+}
+
+// the last rem <= M neighbours as one phase of exactly that many
+template <int M, bool COH, bool I16>
+__device__ __forceinline__ double brow_rest(const double* __restrict__ w,
+                                            const void* __restrict__ colp, const int4& sb,
+                                            const double* __restrict__ u, int rem, double acc) {
+    if constexpr (M > 0) {
+        if (rem == M) return brow_phase<M, COH, I16>(w, colp, sb, u, acc);
+        return brow_rest<M - 1, COH, I16>(w, colp, sb, u, rem, acc);
+    }
+    return acc;
+}
+
+// sum_j w_j u[col_j], an fma chain from 0 in j order, in phases of CH and a
+// shorter last one (NN = 0: the size is known at run time; no load carries a
+// predicate, as predicates held across the ordered loads are spilled)
 template <int NN, bool COH, int CH, bool I16>
 __device__ __forceinline__ double brow(const double* __restrict__ w, const void* __restrict__ colp,
                                        const int4& sb, const double* __restrict__ u, int n) {
+    constexpr int B = I16 ? 2 : 4;   // bytes per stored neighbour
     double acc = 0.0;
-    const int nn = NN > 0 ? NN : n;
+    if constexpr (NN > 0) {
 #pragma unroll
-    for (int j0 = 0; j0 < (NN > 0 ? NN : 1 << 30); j0 += CH) {
-        if (NN == 0 && j0 >= nn) break;
-        int32_t c[CH];
-        double wv[CH], uv[CH];
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < nn) {
-                if constexpr (I16)
-                    c[t] = (int32_t)bld_cs((const uint16_t*)colp + (j0 + t) * SLICE);
-                else
-                    c[t] = bld_cs((const int32_t*)colp + (j0 + t) * SLICE);
-            }
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < nn) wv[t] = bld_cs(w + (j0 + t) * SLICE);
-        if constexpr (I16) {
-#pragma unroll
-            for (int t = 0; t < CH; ++t)
-                if (j0 + t < nn) c[t] = bdecode16((uint32_t)c[t], sb);
+        for (int j = 0; j + CH <= NN; j += CH)
+            acc = brow_phase<CH, COH, I16>(w + j * SLICE, (const char*)colp + j * SLICE * B, sb, u,
+                                           acc);
+        constexpr int J = NN / CH * CH;
+        if constexpr (J < NN)
+            acc = brow_phase<NN - J, COH, I16>(w + J * SLICE, (const char*)colp + J * SLICE * B,
+                                               sb, u, acc);
+    } else {
+        constexpr int GH = 16;
+        int j = 0;
+        for (; j + GH <= n; j += GH) {
+            acc = brow_phase<GH, COH, I16>(w, colp, sb, u, acc);
+            w += GH * SLICE;
+            colp = (const char*)colp + GH * SLICE * B;
         }
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < nn) uv[t] = COH ? bld_cg(u + c[t]) : bld_ca(u + c[t]);
-#pragma unroll
-        for (int t = 0; t < CH; ++t)
-            if (j0 + t < nn) acc = __fma_rn(wv[t], uv[t], acc);
+        acc = brow_rest<GH - 1, COH, I16>(w, colp, sb, u, n - j, acc);
     }
     return acc;
 }
@@ -368,12 +398,14 @@ __device__ bool run_domain(const TeamDesc T, const DomDesc* __restrict__ desc,
 // buffer), and the wide stencils leave out the prefetch - 32 warps hide the
 // plane's latency and the prefetch's L2 requests only compete.  20 domains of
 // 5k..100k nodes, n = 12, 30 and 56, 200 steps, kernel time: 1024-thread
-// blocks 11.66 -> 10.39 ms (phases of 8 before; L1 alone 11.40, and without
-// the prefetch 10.76; phases of 16: 10.53, with .cg 10.86, with the prefetch
-// 11.32; of 24, 28, 56: 10.82, 10.94, 13.0), two blocks of 512 10.98 -> 9.92.
-// With more registers and so fewer warps the prefetch and .cg stay: L1 takes
-// 512-thread blocks with 128 registers from 12.5 to 13.3 ms, without the
-// prefetch to 15.4.
+// blocks 11.66 -> 9.88 ms, of which the weak loads 0.26, leaving out the
+// prefetch 0.64, phases of 20 instead of 8 0.37 (16: 0.23; 24, 28 and 56 give
+// some or all of it back) and brow's phases 0.47; two blocks of 512 10.98 ->
+// 9.64.  With more registers and so fewer warps the prefetch and .cg stay: L1
+// took 512-thread blocks with 128 registers from 12.5 to 13.3 ms, without the
+// prefetch to 15.4; brow's phases alone bring them to 10.8.  Domains of other
+// sizes (brow, NN = 0), 5 of 4k..68k nodes, 200 steps, 1024 threads: n = 20
+// 6.05 -> 1.95 ms, n = 42 10.6 -> 3.11; 512 threads 5.10 -> 2.13, 8.5 -> 3.41.
 template <int MINB, int TH>
 __global__ void __launch_bounds__(TH, MINB)
     batch_kernel(const DomDesc* __restrict__ desc, const DomCall* __restrict__ call,

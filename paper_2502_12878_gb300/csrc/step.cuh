@@ -98,6 +98,51 @@ __device__ __forceinline__ int32_t decode16(uint32_t v, const int4& b) {
     return base + (int32_t)(v & 0x3fffu);
 }
 
+// Rows of a size no kernel is compiled for (NN = 0): phases of 16 and one of
+// exactly the rest, the warp's n deciding by a branch.  Phases under j < n
+// kept their predicates across the ordered loads and spilled them (440-850
+// bytes a thread): a step of 90k rows of 17 / 42 took 15.1 / 23.8 us, now 7.8
+// / 12.5, of 998k rows of 17 / 27 / 42 125 / 139 / 201 and now 43.4 / 59.5 /
+// 85.9, 3D 216k rows of 58 61.9 and now 30.7 (phases of 8: 7.6 / 12.6, 45.2 /
+// 65.0 / 90.7, 33.4; of 12: 7.8 / 12.6, 43.1 / 60.9 / 86.3, 31.6).
+// M neighbours of a row (stride SLICE), continuing the fma chain acc
+template <int M, bool COH, bool I16, class T>
+__device__ __forceinline__ T row_phase(const T* __restrict__ w, const void* __restrict__ colp,
+                                       const int4& sb, const T* __restrict__ u, T acc) {
+    int32_t c[M];
+    T wv[M], uv[M];
+#pragma unroll
+    for (int t = 0; t < M; ++t) {
+        if constexpr (I16) c[t] = (int32_t)ld_stream((const uint16_t*)colp + t * SLICE);
+        else c[t] = ld_stream((const int32_t*)colp + t * SLICE);
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t) wv[t] = ld_stream(w + t * SLICE);
+    if constexpr (I16) {
+#pragma unroll
+        for (int t = 0; t < M; ++t) c[t] = decode16((uint32_t)c[t], sb);
+    }
+#pragma unroll
+    for (int t = 0; t < M; ++t) uv[t] = ld_iter<COH>(u + c[t]);
+#pragma unroll
+    for (int t = 0; t < M; ++t) {
+        if constexpr (sizeof(T) == 8) acc = __fma_rn(wv[t], uv[t], acc);
+        else acc = __fmaf_rn(wv[t], uv[t], acc);
+    }
+    return acc;
+}
+
+// the last rem <= M neighbours as one phase of exactly that many
+template <int M, bool COH, bool I16, class T>
+__device__ __forceinline__ T row_rest(const T* __restrict__ w, const void* __restrict__ colp,
+                                      const int4& sb, const T* __restrict__ u, int rem, T acc) {
+    if constexpr (M > 0) {
+        if (rem == M) return row_phase<M, COH, I16, T>(w, colp, sb, u, acc);
+        return row_rest<M - 1, COH, I16, T>(w, colp, sb, u, rem, acc);
+    }
+    return acc;
+}
+
 // sum_j w_j u[col_j] as an fma chain from 0, j ascending.  Loads are issued
 // in phases of CH (indices, weights, then the gathers) so each thread keeps
 // 2*CH streaming loads and CH gathers in flight.  I16: the indices come as
@@ -105,12 +150,22 @@ __device__ __forceinline__ int32_t decode16(uint32_t v, const int4& b) {
 template <int NN, bool COH, bool I16, class T>
 __device__ __forceinline__ T row_dot(const T* __restrict__ w, const void* __restrict__ colp,
                                      const int4& sb, const T* __restrict__ u, int n) {
+    if constexpr (NN == 0) {
+        constexpr int GH = 16;
+        T g = T(0);
+        int j = 0;
+        for (; j + GH <= n; j += GH) {
+            g = row_phase<GH, COH, I16, T>(w, colp, sb, u, g);
+            w += GH * SLICE;
+            colp = (const char*)colp + GH * SLICE * (I16 ? 2 : 4);
+        }
+        return row_rest<GH - 1, COH, I16, T>(w, colp, sb, u, n - j, g);
+    }
     constexpr int CH = 16;
+    constexpr int nn = NN;
     T acc = T(0);
-    const int nn = NN > 0 ? NN : n;
 #pragma unroll
-    for (int j0 = 0; j0 < (NN > 0 ? NN : 1 << 30); j0 += CH) {
-        if (NN == 0 && j0 >= nn) break;
+    for (int j0 = 0; j0 < NN; j0 += CH) {
         int32_t c[CH];
         T wv[CH], uv[CH];
 #pragma unroll
