@@ -468,23 +468,6 @@ __global__ void __launch_bounds__(STEP_THREADS, NN > 0 ? 4 : 1) power_apply(Step
     }
 }
 
-// single block: norm = sqrt(sum part) in a fixed order; v = y / norm
-__global__ void power_normalize(const double* part, int nparts, const double* y, double* v,
-                                int64_t NI, double* norm_out) {
-    __shared__ double sh[256];
-    double t = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) t += part[i];
-    sh[threadIdx.x] = t;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    double nrm = sqrt(sh[0]);
-    if (threadIdx.x == 0) *norm_out = nrm;
-    for (int64_t p = threadIdx.x; p < NI; p += blockDim.x) v[p] = y[p] / nrm;
-}
-
 __global__ void power_scale(const double* norm, const double* y, double* v, int64_t NI) {
     double nrm = *norm;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
@@ -870,7 +853,6 @@ static int grid_for(const rbffd_plan* p, int per_sm) {
     int64_t cap = (int64_t)device_sm_count() * std::max(1, per_sm);
     return (int)std::max<int64_t>(1, std::min(blocks, cap));
 }
-static int step_grid(const rbffd_plan* p) { return grid_for(p, p->grid_steps); }
 
 // resident blocks of a persistent launch, no more than the slices need
 // (spread plans: one block per SM at most)
