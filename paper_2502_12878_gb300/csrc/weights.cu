@@ -548,10 +548,16 @@ __device__ __forceinline__ void weights_one(const WeightArgs& A, int64_t r, doub
 // which share its FP64 pipe, and three on the others - so equal shares fixed in
 // advance leave three pipes idle while the fourth finishes: 1M stencils, s = 45
 // 94.8 -> 89.9 ms; s = 46 (twelve teams: three on each) 99.7 -> 97.9; s = 18
-// 12.3 -> 12.0.  take_ticket draws the next one (the team's first thread) and is
-// called a stencil ahead, which hides the atomic's latency; share_ticket tells the team.
-__device__ __forceinline__ long long take_ticket(unsigned long long* tickets, int tid) {
-    return tid == 0 ? (long long)atomicAdd(tickets, 1ull) : 0ll;
+// 12.3 -> 12.0.  Every team's first stencil is fixed - were it a ticket too, the
+// teams that start first would hold two while others get none (841 stencils of
+// s = 45 on 1976 teams 264 -> 418 us) - and consecutive ones go to different
+// blocks, so that few stencils spread over all SMs.  take_ticket draws
+// the next one after those (the team's first thread) and is called a stencil
+// ahead, which hides the atomic's latency; share_ticket tells the team.
+__device__ __forceinline__ long long take_ticket(unsigned long long* tickets, int tid,
+                                                 int64_t teams, int64_t total) {
+    if (teams >= total) return (long long)total;   // (the counter is not used, nor set)
+    return tid == 0 ? (long long)teams + (long long)atomicAdd(tickets, 1ull) : 0ll;
 }
 template <int TS>
 __device__ __forceinline__ int64_t share_ticket(long long v, int tid, int team,
@@ -580,12 +586,12 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
     double* G = wsm + (size_t)team * weight_team_doubles(A);
     double* xi = G + (size_t)A.s * A.pitch;
     __shared__ long long s_next[16];
-    long long ticket = take_ticket(tickets, tid);
-    for (;;) {
-        const int64_t r = share_ticket<TS>(ticket, tid, team, s_next);
-        if (r >= A.nc) break;
-        ticket = take_ticket(tickets, tid);
+    const int64_t teams = (int64_t)gridDim.x * (blockDim.x / TS);
+    int64_t r = blockIdx.x + (int64_t)team * gridDim.x;
+    while (r < A.nc) {
+        const long long ticket = take_ticket(tickets, tid, teams, A.nc);
         weights_one<TS, PW>(A, r, G, xi, tid, team, redv, redk, redi, bcast, spiv);
+        r = share_ticket<TS>(ticket, tid, team, s_next);
     }
 }
 
@@ -607,11 +613,10 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
     double* G = wsm + (size_t)team * (size_t)team_doubles;
     __shared__ long long s_next[16];
     const int64_t total = off[ncalls];
-    long long ticket = take_ticket(tickets, tid);
-    for (;;) {
-        const int64_t g = share_ticket<TS>(ticket, tid, team, s_next);
-        if (g >= total) break;
-        ticket = take_ticket(tickets, tid);
+    const int64_t teams = (int64_t)gridDim.x * (blockDim.x / TS);
+    int64_t g = blockIdx.x + (int64_t)team * gridDim.x;
+    while (g < total) {
+        const long long ticket = take_ticket(tickets, tid, teams, total);
         int lo = 0, hi = ncalls - 1;   // last call with off <= g
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -621,6 +626,7 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
         const WeightArgs& A = calls[lo];
         double* xi = G + (size_t)A.s * A.pitch;
         weights_one<TS, PW>(A, g - off[lo], G, xi, tid, team, redv, redk, redi, bcast, spiv);
+        g = share_ticket<TS>(ticket, tid, team, s_next);
     }
 }
 
@@ -779,15 +785,18 @@ static int weights_impl(const double* xyz, int64_t N, int d, const int32_t* idx,
     const int ts = weight_team_size(A.s);
     WeightKernel kern = weight_kernel_for(ts);
     RBFFD_CHECK_CUDA(pick_weight_shape(kern, ts, per_team, &ws));
-    int64_t want = (nc + ws.tpb - 1) / ws.tpb;
-    int64_t grid = std::min<int64_t>(want, (int64_t)sms * ws.per_sm);
+    // (a block a stencil up to what is resident: the first stencils go to different blocks)
+    const int64_t grid = std::min<int64_t>(nc, (int64_t)sms * ws.per_sm);
     Scratch cnt;   // singular stencils, the first of them, the teams' tickets
     RBFFD_CHECK_CUDA(cnt.alloc(3 * sizeof(unsigned long long), s));
-    RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.p, 0, 3 * sizeof(unsigned long long), s));
-    RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.as<unsigned long long>() + 1, 0xff,
-                                     sizeof(unsigned long long), s));
+    if (grid * ws.tpb < nc)   // (else no team takes a ticket)
+        RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.as<unsigned long long>() + 2, 0,
+                                         sizeof(unsigned long long), s));
     kern<<<(unsigned)grid, ws.threads, ws.smem, s>>>(A, cnt.as<unsigned long long>() + 2);
     RBFFD_CHECK_CUDA(cudaGetLastError());
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(unsigned long long), s));
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(cnt.as<unsigned long long>() + 1, 0xff,
+                                     sizeof(unsigned long long), s));
     count_bad<<<sms * 4, 256, 0, s>>>(status, nc, cnt.as<unsigned long long>(),
                                       cnt.as<unsigned long long>() + 1);
     RBFFD_CHECK_CUDA(cudaGetLastError());
@@ -885,8 +894,7 @@ extern "C" int rbffd_weights_batch(int ncalls, const double* const* xyz, const i
         const int ts = weight_team_size(max_s);
         WeightMultiKernel kern = weight_multi_kernel_for(ts);
         RBFFD_CHECK_CUDA(pick_weight_shape(kern, ts, per_team, &ws));
-        const int64_t want = (off.back() + ws.tpb - 1) / ws.tpb;
-        const int64_t grid = std::min<int64_t>(want, (int64_t)sms * ws.per_sm);
+        const int64_t grid = std::min<int64_t>(off.back(), (int64_t)sms * ws.per_sm);
         Scratch tickets;
         RBFFD_CHECK_CUDA(tickets.alloc(sizeof(unsigned long long), s));
         RBFFD_CHECK_CUDA(cudaMemsetAsync(tickets.p, 0, sizeof(unsigned long long), s));
