@@ -193,15 +193,22 @@ __device__ __forceinline__ void link_control(const StepArgs& A, StepCtrl* c, Lin
     }
 }
 
-// poll the entry of slot q until it is of the awaited step
+// poll the entry of slot q until it is of the awaited step.  Blocks leave a run
+// that stopped at different steps, as each learns of the stop at its own time, so
+// the entry's owner may have left before the step that writes it.  Then this block
+// is beyond the stop too and its value no longer matters: the wait also ends, not
+// as a failure, when the stop is known here (the control warp polls it on its own).
 template <class T>
 __device__ __forceinline__ bool link_wait(const unsigned long long* x, int32_t q, unsigned tag,
-                                          T* to, long long spin) {
+                                          T* to, long long spin, const LinkShared& S) {
     T v;
     if (!link_get(x, q, tag, &v)) {
         const long long t0 = clock64();
-        while (!link_get(x, q, tag, &v))
-            if (clock64() - t0 > spin) return false;
+        for (unsigned i = 1; !link_get(x, q, tag, &v); ++i)   // (the rare ends every 16 looks)
+            if ((i & 15u) == 0) {
+                if (S.stop >= 0) break;
+                if (clock64() - t0 > spin) return false;
+            }
     }
     *to = v;
     return true;
@@ -399,14 +406,14 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
         }
         if (npoll > 0 && polls && !have) {
             for (int i = pstart; i < nint; i += pstep)
-                bad = !link_wait(xc, slot_s[i], tag, vc + rows + i, spin) || bad;
+                bad = !link_wait(xc, slot_s[i], tag, vc + rows + i, spin, S) || bad;
             asm volatile("barrier.cta.arrive 2, %0;" ::"r"(hcount) : "memory");
         }
         for (int i = warp; i < nsl; i += NW) {
             if (i >= nin && !have) {
                 if (npoll == 0)
                     for (int j = pstart; j < nint; j += pstep)
-                        bad = !link_wait(xc, slot_s[j], tag, vc + rows + j, spin) || bad;
+                        bad = !link_wait(xc, slot_s[j], tag, vc + rows + j, spin, S) || bad;
                 asm volatile("barrier.cta.sync 2, %0;" ::"r"(hcount) : "memory");
                 have = true;
             }

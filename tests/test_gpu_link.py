@@ -84,6 +84,40 @@ def test_same_bits_as_graph_steps(rb, orc, d, Kg, m, n, order, threads):
     assert _linked(lnk.stats()[3]) or threads == 512 and n >= 56
 
 
+@pytest.mark.parametrize("d,Kg,m,n", [(2, 9, 2, 12), (2, 30, 1, 6), (2, 75, 2, 12), (2, 110, 1, 6)])
+def test_thousands_of_stops(rb, orc, d, Kg, m, n):
+    """Blocks learn of a stop at their own times, and a block that is a step further than its
+    neighbours waits for rows that are never written: it has to find the stop instead of running
+    out of its wait.  Short steps (small n, FP32 too) on 2 to 152 blocks, stopped some 2,000 times
+    by tolerance and 500 by rho_in at every distance from the start."""
+    p = build(orc, d, Kg, m, seed=7, n=n)
+    ref, lnk = _plans(rb, p, 0)
+    f, u0 = T(p.f), T(p.u0)
+    dt = 0.5 * 2.0 / np.abs(p.w).sum(1).max()
+    hist, its = [], []
+    u = u0.clone()
+    for k in range(40):
+        hist.append(ref.solve_explicit(f, u, dt, 1)[2])
+        its.append(u.clone())
+    # the steps whose residual is the smallest so far: where a tolerance above it stops
+    stops = [k for k in range(40) if all(hist[k] < r for r in hist[:k])]
+    v = torch.empty_like(u0)
+    for rep in range(-(-2000 // len(stops))):
+        for k in stops:
+            v.copy_(u0)
+            got = lnk.solve_explicit(f, v, dt, 100000, np.nextafter(hist[k], np.inf))
+            assert got == (rb.RBFFD_OK, k + 1, hist[k])
+            assert torch.equal(v, its[k])
+    assert _linked(lnk.stats()[3])
+    for rho in np.linspace(0.999, 0.5, 25):
+        v.copy_(u0)
+        want = ref.solve_dc(f, v, dt, 0.0, 2, 3000, rho)
+        for rep in range(10):
+            w = u0.clone()
+            assert lnk.solve_dc(f, w, dt, 0.0, 2, 3000, rho) == want
+            assert torch.equal(v, w)
+
+
 def test_nonfinite_and_diverging_runs_end(rb, orc):
     p = build(orc, 2, 80, 2, seed=9)
     ref, lnk = _plans(rb, p, 0)
