@@ -486,7 +486,9 @@ __device__ __forceinline__ void pds_decide(volatile uint8_t* st, const int32_t* 
                 if (in || out) open = false;
             }
             if ((news >> lane) & 1u) st[p] = (acc >> lane) & 1u ? PDS_IN : PDS_OUT;
-            if ((++looks & 1023) == 0 && clock64() - t0 > PDS_SPIN) {
+            // (one lane's clock for the warp: its lanes leave together or not at all)
+            if ((++looks & 1023) == 0 &&
+                __shfl_sync(FULL, clock64() - t0 > PDS_SPIN ? 1 : 0, 0)) {
                 if (lane == 0) atomicCAS(err, 0, 6);
                 break;
             }
