@@ -2253,6 +2253,17 @@ extern "C" int rbffd_solve_dc(rbffd_plan* p, const double* f, double* u, double 
     return status;
 }
 
+// the Neumann nodes' values after `steps` steps, to the caller's u (the interior
+// is there already: scatter_result)
+static int neumann_result(rbffd_plan* p, long long steps, double* u, cudaStream_t s) {
+    if (p->NN == 0) return RBFFD_OK;
+    neumann_out<<<device_sm_count() * 2, 256, 0, s>>>(p->nslot, p->u[steps & 1], p->perm, p->NN, u);
+    p->last_launches += 1;
+    RBFFD_CHECK_CUDA(cudaGetLastError());
+    RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
+    return RBFFD_OK;
+}
+
 extern "C" int rbffd_solve_explicit(rbffd_plan* p, const double* f, double* u, double dt,
                                     int64_t max_steps, double tol, int precision,
                                     int64_t* h_steps_out, double* h_res_out, void* stream) {
@@ -2276,14 +2287,8 @@ extern "C" int rbffd_solve_explicit(rbffd_plan* p, const double* f, double* u, d
     double R = 0.0;
     int done = 0;
     st = run_steps(p, MODE_SWEEP64, dt, tol, max_steps, s, &steps, &R, &done, u);
+    if (!st) st = neumann_result(p, steps, u, s);
     if (st) return st;
-    if (p->NN > 0) {
-        neumann_out<<<device_sm_count() * 2, 256, 0, s>>>(p->nslot, p->u[steps & 1], p->perm,
-                                                          p->NN, u);
-        p->last_launches += 1;
-        RBFFD_CHECK_CUDA(cudaGetLastError());
-        RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
-    }
     if (h_steps_out) *h_steps_out = steps;
     if (h_res_out) *h_res_out = R;
     if (max_steps == 0) return RBFFD_NOT_CONVERGED;
@@ -2564,14 +2569,21 @@ extern "C" int rbffd_solve_record(rbffd_plan* p, const double* f, double* u, dou
                                                    ckpt + k / seg * p->N);
         RBFFD_CHECK_CUDA(cudaGetLastError());
         const int64_t m = std::min(seg, K - k);
+        // the result behind the last segment, or behind the one that does not get through
         st = run_steps(p, MODE_SWEEP64, dt, 0.0, m, s, &steps, &R, &done,
                        k + m == K ? u : nullptr);
         if (st) return st;
-        if (done != DONE_CAP) {
+        if (done != DONE_CAP && k + m < K) {
             scatter_u<<<sms * 8, 256, 0, s>>>(p->u[steps & 1], p->perm, p->NI, u);
-            cudaStreamSynchronize(s);
-            return done_status(done);
+            p->last_launches += 1;
+            RBFFD_CHECK_CUDA(cudaGetLastError());
+            RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
         }
+        if (done != DONE_CAP || k + m == K) {
+            st = neumann_result(p, steps, u, s);
+            if (st) return st;
+        }
+        if (done != DONE_CAP) return done_status(done);
         // a run starts from u[0], and its boundary (and Neumann) slots are in both
         if (k + m < K && (m & 1))
             RBFFD_CHECK_CUDA(cudaMemcpyAsync(p->u[0], p->u[1], sizeof(double) * p->N,

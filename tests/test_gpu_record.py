@@ -1,11 +1,12 @@
 """Recorded runs (rbffd_solve_record) against solves of one segment after another, bit for bit:
 every launch family, segments that divide K or not, records of every step or of segments, none at
-all; the same divergence verdict; and the differentiable solve through either."""
+all; the same divergence verdict; plans with Neumann nodes; and the differentiable solve through
+either."""
 import numpy as np
 import pytest
 
 import rbffd_inputs as gen
-from oracle_problem import build
+from oracle_problem import build, build_mixed
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -65,6 +66,33 @@ def test_record_equals_segment_solves(rb, orc, Kg, m, flags):
             except rb.RbffdError as e:
                 got.append(e.code)
         assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("flags", [0, 64])
+def test_record_with_neumann_nodes(rb, orc, flags):
+    mp = build_mixed(orc, 2, 24, 2, seed=3)
+    p = mp.base
+    plan = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w), flags)
+    plan.set_neumann(T(mp.nnode), T(mp.nidx), T(mp.nw), T(mp.g + 0.25))
+    dt = 0.5 * 2.0 / np.abs(p.w).sum(1).max()
+    f = T(p.f)
+    for K, seg, scale in ((20, 5, 1), (21, 4, 1), (1, 3, 1), (30, 7, 1e6)):
+        u, v, kept, code = T(p.u0), T(p.u0), [], [0, 0]
+        rows = -(-K // seg)
+        ck = torch.zeros((rows, p.N), dtype=torch.float64, device="cuda")
+        try:
+            for k in range(0, K, seg):
+                kept.append(u.clone())
+                plan.solve_explicit(f, u, scale * dt, min(seg, K - k))
+        except rb.RbffdError as e:
+            code[0] = e.code
+        try:
+            assert plan.solve_record(f, v, scale * dt, K, seg, ck) == seg
+        except rb.RbffdError as e:
+            code[1] = e.code
+        assert code[0] == code[1] and (scale == 1 or code[0] != 0)
+        assert torch.equal(u, v)
+        assert torch.equal(ck[:len(kept)], torch.stack(kept))
 
 
 def test_differentiable_solve_keeps_its_bits(rb, orc):
