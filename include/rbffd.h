@@ -529,7 +529,10 @@ RBFFD_API int rbffd_batch_domain_times(const rbffd_batch* batch, double* h_start
  * Eq. 7 (cfl) bounds dt by h^2/(2d) for regular nodes only; here the bound is
  * 2 / (safety * rho), rho the spectral radius of the interior block W_II
  * estimated by `iters` power iterations from v0 [NI] (plan's interior order):
- * y = W_II v, rho = ||y||_2, v = y / rho.
+ * y = W_II v, rho = ||y||_2, v = y / rho.  On plans without Neumann nodes the
+ * iterations run in cooperative launches, scaled by powers of two instead of
+ * 1 / rho; their waits have rbffd_plan_set_wait's limit, and where one runs out
+ * the estimate is made again by launches that do not wait for each other.
  */
 RBFFD_API int rbffd_stable_dt(rbffd_plan* plan, const double* v0, int iters, double safety,
                     double* h_dt_out, double* h_rho_out, void* stream);

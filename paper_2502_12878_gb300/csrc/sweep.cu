@@ -526,6 +526,7 @@ power_persist(StepArgs A, StepCtrl* c, long long iters, double* part) {
     const int64_t nw = (int64_t)gridDim.x * (STEP_THREADS / 32);
     const long long lim = ((volatile StepCtrl*)c)->spin_limit;
     const long long spin = lim > 0 ? lim : (long long)SPIN_LIMIT_CYCLES;
+    const unsigned held = (unsigned)((volatile StepCtrl*)c)->held;
     for (long long k = 0; k < iters; ++k) {
         const double* v = (k & 1) ? A.u1 : A.u0;
         double* y = (k & 1) ? A.u0 : A.u1;
@@ -573,7 +574,7 @@ power_persist(StepArgs A, StepCtrl* c, long long iters, double* part) {
             if (blockIdx.x == 0) st_relaxed(&c->res[(k + 2) % 3], 0ull);
             red_max_relaxed(&c->res[(k + 1) % 3], m);
             red_add_release(&c->arrivals, 1ull);
-            const unsigned long long target = (unsigned long long)(k + 1) * gridDim.x;
+            const unsigned long long target = (unsigned long long)(k + 1) * gridDim.x + held;
             const long long t0 = clock64();
             while (ld_acquire(&c->arrivals) < target)
                 if (clock64() - t0 > spin) {
@@ -874,8 +875,20 @@ static int persistent_grid(StepFn fn, const rbffd_plan* p) {
 // test of the timeout path, rbffd_plan_set_wait)
 __global__ void ctrl_set(StepCtrl* c, const StepCtrl v) { *c = v; }
 
+// the same behind a run whose outcome nobody has read yet: one that did not take
+// all its steps is kept in *bad (its first such code), and the new run gets none
+__global__ void ctrl_next(StepCtrl* c, const StepCtrl v, int* bad) {
+    const int was = c->done;
+    if (was != DONE_CAP && *bad == 0) *bad = was ? was : DONE_TIMEOUT;
+    *c = v;
+    if (*bad) {
+        c->max_steps = 0;
+        c->done = DONE_CAP;
+    }
+}
+
 static int ctrl_reset(rbffd_plan* p, double dt, double tol, long long max_steps, cudaStream_t s,
-                      int held = 0) {
+                      int held = 0, int* bad = nullptr) {
     StepCtrl h;
     memset(&h, 0, sizeof(h));
     h.max_steps = max_steps;
@@ -884,7 +897,8 @@ static int ctrl_reset(rbffd_plan* p, double dt, double tol, long long max_steps,
     h.done = max_steps <= 0 ? DONE_CAP : DONE_RUNNING;
     h.held = held;
     h.spin_limit = p->spin_limit;
-    ctrl_set<<<1, 1, 0, s>>>(p->ctrl, h);
+    if (bad) ctrl_next<<<1, 1, 0, s>>>(p->ctrl, h, bad);
+    else ctrl_set<<<1, 1, 0, s>>>(p->ctrl, h);
     RBFFD_CHECK_CUDA(cudaGetLastError());
     return RBFFD_OK;
 }
@@ -2392,12 +2406,13 @@ __global__ void link_norms(const double* __restrict__ y, const unsigned long lon
 // with c the power of two just below 1 / max row sum of |W|, so no component
 // grows, at most POWER_CHUNK iterations a launch, between which the vector is
 // scaled back (exactly).  *done false where the plan does not fit it or has
-// rows of no size.  200 iterations against the persistent launch: 10k rows, n = 12
+// rows of no size, or, with *late, where a wait of any of the launches ran out (its
+// vector is then not written, and the launches behind it do nothing).  200 iterations against the persistent launch: 10k rows, n = 12
 // 0.81 -> 0.48 ms; 90k, n = 30 2.06 -> 1.32, n = 24 2.96 -> 1.12.
 static constexpr int POWER_CHUNK = 64;
 
 static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int iters,
-                        double* rho, bool* done, cudaStream_t s) {
+                        double* rho, bool* done, bool* late, cudaStream_t s) {
     if (iters < 2 || !(p->flags & (RBFFD_LAUNCH_AUTO | RBFFD_LAUNCH_RESIDENT)))
         return RBFFD_OK;
     int st = build_link(p, s);
@@ -2415,7 +2430,8 @@ static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int
     constexpr int NP = 512;   // partial sums
     double* part = p->scratch + 8;
     unsigned long long* mx = reinterpret_cast<unsigned long long*>(p->scratch);   // [0] W, [1] v
-    RBFFD_CHECK_CUDA(cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned long long), s));
+    int* bad = reinterpret_cast<int*>(mx + 2);   // first outcome of a launch that fell short
+    RBFFD_CHECK_CUDA(cudaMemsetAsync(mx, 0, 3 * sizeof(unsigned long long), s));
     RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[0], 0, sizeof(double) * p->N, s));
     RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[1], 0, sizeof(double) * p->N, s));
     gather_f<<<sms * 8, 256, 0, s>>>(v0, p->row_of_slot, p->NI, p->u[0]);
@@ -2435,7 +2451,8 @@ static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int
         // the last launch has at least two iterations: its last two iterates are summed
         const int k = left <= POWER_CHUNK ? left : left == POWER_CHUNK + 1 ? POWER_CHUNK - 1
                                                                            : POWER_CHUNK;
-        if ((st = ctrl_reset(p, sc, 0.0, k, s))) return st;
+        if ((st = ctrl_reset(p, sc, 0.0, k, s, p->held_arrivals, left < iters ? bad : nullptr)))
+            return st;
         StepArgs A = A0;
         A.u0 = p->u[cur];
         A.u1 = p->u[cur ^ 1];
@@ -2465,21 +2482,24 @@ static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int
                                   p->NI, part, part + NP);
     power_rho<<<1, 256, 0, s>>>(part + 2 * NP, NP, part, NP, part + NP, NP, psc, p->scratch);
     RBFFD_CHECK_CUDA(cudaGetLastError());
-    int how = 0;
+    int how = 0, before = 0;
+    double out[3];   // the radius, and `bad` two words on
     RBFFD_CHECK_CUDA(cudaMemcpyAsync(&how, &p->ctrl->done, sizeof(int), cudaMemcpyDeviceToHost,
                                      s));
-    RBFFD_CHECK_CUDA(cudaMemcpyAsync(rho, p->scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
+    RBFFD_CHECK_CUDA(cudaMemcpyAsync(out, p->scratch, sizeof(out), cudaMemcpyDeviceToHost, s));
     RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
-    if (how == DONE_TIMEOUT) return done_status(how);
-    if (how != DONE_CAP) *rho = NAN;   // not finite on the way
-    *done = true;
+    memcpy(&before, out + 2, sizeof(before));
+    if (before) how = before;
+    *late = how == DONE_TIMEOUT;
+    *rho = how == DONE_CAP ? out[0] : NAN;   // (else not finite on the way)
+    *done = !*late;
     return RBFFD_OK;
 }
 
 // the power iteration in one cooperative launch; *done false where the device
-// cannot hold the grid at once
+// cannot hold the grid at once, or, with *late, where a wait ran out
 static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int iters,
-                        double* rho, bool* done, cudaStream_t s) {
+                        double* rho, bool* done, bool* late, cudaStream_t s) {
     const int sms = device_sm_count();
     typedef void (*PowFn)(StepArgs, StepCtrl*, long long, double*);
     PowFn pf;
@@ -2494,7 +2514,7 @@ static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int 
     const int nparts = 1024;
     if (2 * grid + 1 > 2 * nparts) return RBFFD_OK;   // scratch holds 4096 partial sums
     double* part = p->scratch + 8;
-    int st = ctrl_reset(p, 0.0, 0.0, iters, s);
+    int st = ctrl_reset(p, 0.0, 0.0, iters, s, p->held_arrivals);
     if (st) return st;
     RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[0], 0, sizeof(double) * p->N, s));
     RBFFD_CHECK_CUDA(cudaMemsetAsync(p->u[1], 0, sizeof(double) * p->N, s));
@@ -2522,8 +2542,8 @@ static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int 
                                      cudaMemcpyDeviceToHost, s));
     RBFFD_CHECK_CUDA(cudaMemcpyAsync(rho, p->scratch, sizeof(double), cudaMemcpyDeviceToHost, s));
     RBFFD_CHECK_CUDA(cudaStreamSynchronize(s));
-    if (stopped == DONE_TIMEOUT) return done_status(DONE_TIMEOUT);
-    *done = true;
+    *late = stopped == DONE_TIMEOUT;
+    *done = !*late;
     return RBFFD_OK;
 }
 
@@ -2599,10 +2619,12 @@ extern "C" int rbffd_stable_dt(rbffd_plan* p, const double* v0, int iters, doubl
     cudaStream_t s = as_stream(stream);
     StepArgs A = make_args(p);
     double rho = 0.0;
-    bool done = false;
+    // the forms whose blocks wait for each other, unless a wait ran out (`late`): the
+    // launches of the stepwise form only queue
+    bool done = false, late = false;
     if (p->NN == 0) {   // (the Neumann update between iterations needs launches of its own)
-        int st = power_linked(p, A, v0, iters, &rho, &done, s);
-        if (!st && !done) st = power_launch(p, A, v0, iters, &rho, &done, s);
+        int st = power_linked(p, A, v0, iters, &rho, &done, &late, s);
+        if (!st && !done && !late) st = power_launch(p, A, v0, iters, &rho, &done, &late, s);
         if (st) return st;
     }
     if (!done) {

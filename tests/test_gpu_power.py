@@ -48,3 +48,18 @@ def test_radius_equals_the_oracles(rb, orc, d, Kg, m, n, flags):
     for bad in (np.zeros(p.NI), np.full(p.NI, np.nan), v0 * 1e-200, v0 * 1e200):
         with pytest.raises(rb.RbffdError):
             plan.stable_dt(T(bad), 5)
+
+
+@pytest.mark.parametrize("n,flags", [(12, 0), (12, 64), (17, 64), (30, 128)])
+def test_waits_that_run_out_do_not_change_the_radius(rb, orc, n, flags):
+    """Withheld arrivals and decisions, and limits about as long as a wait takes, so that any
+    launch of the linked form may fall short: the radius is the same."""
+    p = build(orc, 2, 100, 2 if n < 30 else 4, seed=17, n=n)
+    plan = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w), flags, 3)
+    v0 = gen.random_vector(p.NI, 5)
+    for iters in (1, 2, 65, 200):
+        rho = orc.power_rho(p.w, p.idx, p.interior, p.N, v0, iters)
+        waits = [(20.0, 1), (0.0, 0)] + [(ms, 0) for ms in (2e-4, 5e-4, 1e-3, 2e-3, 4e-3) * 4]
+        for wait in waits:
+            plan.set_wait(*wait)
+            assert abs(plan.stable_dt(T(v0), iters, 1.05)[1] - rho) <= 1e-9 * rho, wait
