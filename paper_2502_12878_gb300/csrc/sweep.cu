@@ -2367,26 +2367,49 @@ __global__ void row_abs_max(const double* __restrict__ w64, int64_t NI, int64_t 
     if (threadIdx.x == 0) red_max_relaxed(out, m);
 }
 
-// v <- 2^-e v with 2^e <= max < 2^(e+1) (bits in *mx; 0, subnormal or not finite: as it is)
-__global__ void scale_to_one(double* v, int64_t NI, const unsigned long long* mx) {
-    const unsigned ex = (unsigned)(*mx >> 52);
-    if (ex < 1u || ex > 2045u) return;
-    const double sc = bitsd((unsigned long long)(2046u - ex) << 52);
+// the power of two that brings a maximum m (IEEE bits) into [1, 2); 1 where m is
+// 0, subnormal or not finite
+__device__ __forceinline__ double to_one(unsigned long long m) {
+    const unsigned ex = (unsigned)(m >> 52);
+    return bitsd(ex >= 1u && ex <= 2045u ? (unsigned long long)(2046u - ex) << 52
+                                         : 0x3ff0000000000000ull);
+}
+
+// A maximum that a launch of the linked power iteration has brought from [1, 2)
+// below 2^-900 is too close to what a double holds (its smaller components may be
+// gone): *bad, unless an earlier outcome is there
+static constexpr int POWER_SMALL = -1;
+__device__ __forceinline__ void power_check(unsigned long long m, int* bad) {
+    if (bad && blockIdx.x == 0 && threadIdx.x == 0 && (unsigned)(m >> 52) < 1023u - 900u &&
+        *bad == 0)
+        *bad = POWER_SMALL;
+}
+
+// v <- 2^-e v with 2^e <= max < 2^(e+1) (bits in *mx)
+__global__ void scale_to_one(double* v, int64_t NI, const unsigned long long* mx, int* bad) {
+    power_check(*mx, bad);
+    const double sc = to_one(*mx);
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
          p += (int64_t)gridDim.x * blockDim.x)
         v[p] = __dmul_rn(v[p], sc);
 }
 
-// partial sums of squares of y (s1) and of the ring's iterate x (s0)
+// partial sums of squares of y (s1, its maximum's bits in *mx) and of the ring's
+// iterate x before it (s0), both scaled by the power of two that brings y's
+// maximum to 1: y's own scale is rho / (max row sum) to the power of the iterations
 __global__ void link_norms(const double* __restrict__ y, const unsigned long long* __restrict__ x,
-                           int64_t NI, double* s0, double* s1) {
+                           int64_t NI, const unsigned long long* mx, int* bad, double* s0,
+                           double* s1) {
     __shared__ double sh[2][256];
+    power_check(*mx, bad);
+    const double sc = to_one(*mx);
     double a = 0.0, b = 0.0;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < NI;
          p += (int64_t)gridDim.x * blockDim.x) {
-        const double u = bitsd((x[2 * p] & 0xffffffffull) | (x[2 * p + 1] << 32));
+        const double u = __dmul_rn(bitsd((x[2 * p] & 0xffffffffull) | (x[2 * p + 1] << 32)), sc);
+        const double t = __dmul_rn(y[p], sc);
         a = __fma_rn(u, u, a);
-        b = __fma_rn(y[p], y[p], b);
+        b = __fma_rn(t, t, b);
     }
     sh[0][threadIdx.x] = a;
     sh[1][threadIdx.x] = b;
@@ -2406,7 +2429,9 @@ __global__ void link_norms(const double* __restrict__ y, const unsigned long lon
 // with c the power of two just below 1 / max row sum of |W|, so no component
 // grows, at most POWER_CHUNK iterations a launch, between which the vector is
 // scaled back (exactly).  *done false where the plan does not fit it or has
-// rows of no size, or, with *late, where a wait of any of the launches ran out (its
+// rows of no size, where the vector shrinks too far in one launch (below 2^-900: rho
+// less than 6e-5 of the largest row sum; the persistent launch scales every
+// iteration) or is not finite, or, with *late, where a wait of any of the launches ran out (its
 // vector is then not written, and the launches behind it do nothing).  200 iterations against the persistent launch: 10k rows, n = 12
 // 0.81 -> 0.48 ms; 90k, n = 30 2.06 -> 1.32, n = 24 2.96 -> 1.12.
 static constexpr int POWER_CHUNK = 64;
@@ -2438,7 +2463,7 @@ static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int
     row_abs_max<<<sms * 4, 256, 0, s>>>(p->w64, p->NI, p->nslices, p->n, mx);
     vec_max<<<sms, 256, 0, s>>>(p->u[0], p->NI, mx + 1);
     norm_partials<<<NP, 256, 0, s>>>(p->u[0], p->NI, part + 2 * NP);
-    scale_to_one<<<sms, 256, 0, s>>>(p->u[0], p->NI, mx + 1);
+    scale_to_one<<<sms, 256, 0, s>>>(p->u[0], p->NI, mx + 1, nullptr);
     RBFFD_CHECK_CUDA(cudaGetLastError());
     unsigned long long wmax = 0;
     RBFFD_CHECK_CUDA(cudaMemcpyAsync(&wmax, mx, sizeof(wmax), cudaMemcpyDeviceToHost, s));
@@ -2469,17 +2494,15 @@ static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int
         left -= k;
         cur ^= k & 1;
         last = k;
-        if (left > 0) {
-            RBFFD_CHECK_CUDA(cudaMemsetAsync(mx + 1, 0, sizeof(unsigned long long), s));
-            vec_max<<<sms, 256, 0, s>>>(p->u[cur], p->NI, mx + 1);
-            scale_to_one<<<sms, 256, 0, s>>>(p->u[cur], p->NI, mx + 1);
-        }
+        RBFFD_CHECK_CUDA(cudaMemsetAsync(mx + 1, 0, sizeof(unsigned long long), s));
+        vec_max<<<sms, 256, 0, s>>>(p->u[cur], p->NI, mx + 1);
+        if (left > 0) scale_to_one<<<sms, 256, 0, s>>>(p->u[cur], p->NI, mx + 1, bad);
     }
     // || y_K || / (sc || y_{K-1} ||): the result and the iterate before it in the ring
     double* psc = part + 3 * NP;
     RBFFD_CHECK_CUDA(cudaMemcpyAsync(psc, &sc, sizeof(sc), cudaMemcpyHostToDevice, s));
     link_norms<<<NP, 256, 0, s>>>(p->u[cur], p->lk_x + (size_t)((last - 1) % LINK_RING) * 2 * p->NI,
-                                  p->NI, part, part + NP);
+                                  p->NI, mx + 1, bad, part, part + NP);
     power_rho<<<1, 256, 0, s>>>(part + 2 * NP, NP, part, NP, part + NP, NP, psc, p->scratch);
     RBFFD_CHECK_CUDA(cudaGetLastError());
     int how = 0, before = 0;
@@ -2491,8 +2514,8 @@ static int power_linked(rbffd_plan* p, const StepArgs& A0, const double* v0, int
     memcpy(&before, out + 2, sizeof(before));
     if (before) how = before;
     *late = how == DONE_TIMEOUT;
-    *rho = how == DONE_CAP ? out[0] : NAN;   // (else not finite on the way)
-    *done = !*late;
+    *rho = out[0];
+    *done = how == DONE_CAP && *rho > 0.0 && isfinite(*rho);
     return RBFFD_OK;
 }
 

@@ -63,3 +63,20 @@ def test_waits_that_run_out_do_not_change_the_radius(rb, orc, n, flags):
         for wait in waits:
             plan.set_wait(*wait)
             assert abs(plan.stable_dt(T(v0), iters, 1.05)[1] - rho) <= 1e-9 * rho, wait
+
+
+@pytest.mark.parametrize("flags", [0, 64, 2])
+@pytest.mark.parametrize("big", [1e3, 1e5, 1e8, 1e40])
+def test_radius_far_below_the_row_sums(rb, orc, flags, big):
+    """A huge weight on a boundary node leaves W_II, and so the radius, as it was, but not the
+    largest row sum, by which the linked launch scales its iterations."""
+    p = build(orc, 2, 60, 2, seed=17, n=12)
+    row = next(r for r in range(p.NI) if p.is_bnd[p.idx[r]].any())
+    w = p.w.copy()
+    j = int(np.nonzero(p.is_bnd[p.idx[row]])[0][0])
+    w[row, j] = big * np.abs(p.w).sum(1).max()
+    plan = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(w), flags, 3)
+    v0 = gen.random_vector(p.NI, 5)
+    for iters in (2, 8, 64, 128, 200, 256):
+        rho = orc.power_rho(p.w, p.idx, p.interior, p.N, v0, iters)
+        assert abs(plan.stable_dt(T(v0), iters, 1.05)[1] - rho) <= 1e-9 * rho
