@@ -429,6 +429,10 @@ RBFFD_API int rbffd_solve_explicit(rbffd_plan* plan, const double* f, double* u,
 RBFFD_API int rbffd_solve_record(rbffd_plan* plan, const double* f, double* u, double dt,
                                  int64_t K, int64_t seg, double* ckpt, int64_t ckpt_rows,
                                  int64_t* h_every_out, void* stream);
+/* whether rbffd_solve_record on this plan can keep every iterate as it runs
+ * (*h_all 1), so that a caller need not hold room for iterates that will not
+ * come.  Tunes the plan's FP64 sweep as its first solve would. */
+RBFFD_API int rbffd_plan_records(rbffd_plan* plan, int* h_all, void* stream);
 
 /*
  * rbffd_plan_stats - what the last solve on this plan did (host outputs, may

@@ -60,7 +60,7 @@ EXPORTED = [
     "rbffd_nodes_pds", "rbffd_nodes_pds_cap", "rbffd_weights_batch", "rbffd_transpose",
     "rbffd_plan_set_wait", "rbffd_fp64_fma_rate", "rbffd_plan_set_resident_halo",
     "rbffd_plan_set_block",
-    "rbffd_transpose_layout", "rbffd_solve_record",
+    "rbffd_transpose_layout", "rbffd_solve_record", "rbffd_plan_records",
 ]
 RBFFD_KNN_NOALLOC_MAX_NODES = 262144
 KEEP_ITERATES = 256 << 20   # bytes of iterates a differentiable solve may keep whole
@@ -102,6 +102,7 @@ def lib():
         "rbffd_plan_perm": (I, [P, P, P]),
         "rbffd_solve_explicit": (I, [P, P, P, D, I64, D, I, PI64, PD, P]),
         "rbffd_solve_record": (I, [P, P, P, D, I64, I64, P, I64, PI64, P]),
+        "rbffd_plan_records": (I, [P, ctypes.POINTER(I), P]),
         "rbffd_solve_dc": (I, [P, P, P, D, D, I64, I64, D, PI64, PI64, PD, P]),
         "rbffd_plan_set_dc": (I, [P, I64, D]),
         "rbffd_stable_dt": (I, [P, P, I, D, PD, PD, P]),
@@ -436,6 +437,12 @@ class Plan:
                                         ctypes.byref(every), _stream(self.device)))
         return every.value
 
+    def records_all(self):
+        """Whether ``solve_record`` can keep every iterate as it runs."""
+        out = ctypes.c_int(0)
+        _check(lib().rbffd_plan_records(self.handle, ctypes.byref(out), _stream(self.device)))
+        return bool(out.value)
+
     def adjoint_w(self, f, ckpt, every, dLdu, K, dt):
         """Backward pass with the weight gradient from checkpoints ckpt [nseg, N] (caller
         order, u^0, u^every, ...) and dLdu = dL/du^K [N].
@@ -671,14 +678,16 @@ class ExplicitSolver:
     ``solver(f, g, w)`` returns u^K [N] from u^0 = 0 inside and g on the boundary
     (``g`` in the order of the boundary nodes, ascending).  Gradients flow to f, g
     and (if it requires grad) the weights w [NI, n].  For the weight gradient the
-    forward keeps every ``every``-th iterate (default ceil(sqrt(K))), from which the
-    backward replays each segment, or, where they take no more than KEEP_ITERATES
-    bytes and the plan can keep them as it runs, all of them."""
+    forward keeps every ``every``-th iterate, from which the backward replays each
+    segment.  Where ``every`` is not given it is ceil(sqrt(K)), or 1 (nothing is
+    replayed) where all iterates take no more than KEEP_ITERATES bytes and the plan
+    can keep them as it runs."""
 
     def __init__(self, xyz, is_bnd, interior, idx, K, dt, every=None, flags=0):
         self.xyz, self.is_bnd = xyz, is_bnd
         self.interior, self.idx = interior, idx
         self.K, self.dt = int(K), float(dt)
+        self.keep_all = not every   # if they are small: the caller set no spacing
         self.every = int(every) if every else max(1, math.ceil(math.sqrt(max(self.K, 1))))
         self.flags = flags
         self.bnd = torch.nonzero(is_bnd).flatten()
@@ -707,11 +716,12 @@ class RBFFDExplicit(torch.autograd.Function):
         plan = solver.plan(w)
         u = torch.zeros(solver.N, dtype=torch.float64, device=f.device)
         u[solver.bnd] = g
-        # without a weight gradient the backward needs no iterates; with one, all of them
-        # where they are small (nothing is replayed then), else every `every`-th
+        # without a weight gradient the backward needs no iterates; with one, every
+        # `every`-th, or all of them (see ExplicitSolver)
         rows, every, ckpt = -(-solver.K // solver.every), solver.every, None
         if ctx.needs_input_grad[2] and solver.K > 0:
-            if solver.K * solver.N * 8 <= KEEP_ITERATES:
+            if (solver.keep_all and solver.K * solver.N * 8 <= KEEP_ITERATES
+                    and plan.records_all()):
                 rows = solver.K
             ckpt = torch.empty((rows, solver.N), dtype=torch.float64, device=f.device)
         if solver.K > 0:

@@ -2570,6 +2570,18 @@ static int power_launch(rbffd_plan* p, const StepArgs& A, const double* v0, int 
     return RBFFD_OK;
 }
 
+// whether a recorded run keeps its iterates in the one launch that makes them
+static bool records_as_it_runs(const rbffd_plan* p) { return p->persist[0] && p->link[0]; }
+
+extern "C" int rbffd_plan_records(rbffd_plan* p, int* h_all, void* stream) {
+    clear_error();
+    RBFFD_ARG(p && h_all, "rbffd_plan_records: NULL argument");
+    const int st = prepare_mode(p, MODE_SWEEP64, 1.0, 0.0, 0, as_stream(stream));
+    if (st) return st;
+    *h_all = records_as_it_runs(p) ? 1 : 0;
+    return RBFFD_OK;
+}
+
 extern "C" int rbffd_solve_record(rbffd_plan* p, const double* f, double* u, double dt, int64_t K,
                                   int64_t seg, double* ckpt, int64_t ckpt_rows,
                                   int64_t* h_every_out, void* stream) {
@@ -2589,7 +2601,7 @@ extern "C" int rbffd_solve_record(rbffd_plan* p, const double* f, double* u, dou
     long long steps = 0;
     double R = 0.0;
     int done = 0;
-    if (p->persist[0] && p->link[0]) {
+    if (records_as_it_runs(p)) {
         // one run, recorded by the launch itself: every step where that fits
         RecordTo rec;
         rec.rec = ckpt;

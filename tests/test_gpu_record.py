@@ -115,3 +115,18 @@ def test_differentiable_solve_keeps_its_bits(rb, orc):
         res.append([u.detach(), *grads, gf])
     for r in res[1:]:
         assert all(torch.equal(a, b) for a, b in zip(r, res[0]))
+
+
+def test_memory_of_a_differentiable_solve(rb, orc):
+    """A caller's spacing bounds the iterates kept; so does a plan that cannot keep them all."""
+    p = build(orc, 2, 70, 4, seed=33)
+    dt = 0.5 * 2.0 / np.abs(p.w).sum(1).max()
+    bnd = p.is_bnd.astype(bool)
+    K = 23
+    for flags, every, rows in ((0, None, 5), (0, 4, 6), (64, 4, 6), (64, 1, K), (64, None, K)):
+        s = rb.ExplicitSolver(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), K, dt, every, flags)
+        f, g, w = (T(a).requires_grad_(True) for a in (p.f, p.u0[bnd], p.w))
+        u = s(f, g, w)
+        kept = u.grad_fn.saved_tensors[1]
+        assert kept.shape == (rows, p.N)
+        assert kept.untyped_storage().nbytes() == rows * p.N * 8
