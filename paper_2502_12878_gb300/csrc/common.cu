@@ -4,7 +4,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -39,75 +38,6 @@ cudaError_t allow_smem(const void* fn, size_t bytes) {
     if (bytes > (size_t)std::max(0, most)) return cudaErrorInvalidValue;
     if (a.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-}
-
-// ----------------------------------------------------------- memory pool
-// A pool lives as long as its device's context: after a cudaDeviceReset the
-// context's id is another one, and a new pool is made (the old one went with
-// its context).
-namespace {
-struct Pools {
-    static constexpr int MAX_DEV = 64;
-    std::mutex mu;
-    cudaMemPool_t pool[MAX_DEV] = {};
-    unsigned long long ctx[MAX_DEV] = {};
-    typedef int (*CtxGetId)(void*, unsigned long long*);
-    CtxGetId ctx_id = nullptr;
-    bool looked = false;
-    ~Pools() {
-        for (int d = 0; d < MAX_DEV; ++d)
-            if (pool[d]) cudaMemPoolDestroy(pool[d]);   // (an error when CUDA has shut down)
-    }
-    // the current device's pool; null where there can be none
-    cudaMemPool_t get() {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return nullptr;
-        std::lock_guard<std::mutex> lock(mu);
-        if (!looked) {
-            looked = true;
-            void* fn = nullptr;
-            cudaDriverEntryPointQueryResult found;
-            if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault,
-                                                 &found) == cudaSuccess &&
-                found == cudaDriverEntryPointSuccess)
-                ctx_id = (CtxGetId)fn;
-        }
-        unsigned long long id = 0;
-        cudaSetDevice(dev);   // makes the device's context current in this thread
-        if (!ctx_id || ctx_id(nullptr, &id) != 0) return nullptr;
-        if (pool[dev] && ctx[dev] == id) return pool[dev];
-        cudaMemPoolProps props;
-        memset(&props, 0, sizeof(props));
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t made = nullptr;
-        unsigned long long keep = POOL_KEEP;
-        if (cudaMemPoolCreate(&made, &props) != cudaSuccess ||
-            cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        pool[dev] = made;
-        ctx[dev] = id;
-        return made;
-    }
-};
-Pools g_pools;
-}  // namespace
-
-cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
-    cudaMemPool_t pool = g_pools.get();
-    if (!pool) return cudaMallocAsync(p, bytes, s);
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    if (e == cudaErrorMemoryAllocation) {   // with what the pool keeps given back
-        cudaGetLastError();
-        cudaStreamSynchronize(s);
-        cudaMemPoolTrimTo(pool, 0);
-        e = cudaMallocFromPoolAsync(p, bytes, pool, s);
-    }
-    return e;
 }
 
 // ------------------------------------------------------------------- scans

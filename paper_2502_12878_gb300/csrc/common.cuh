@@ -10,6 +10,7 @@
 #include <string>
 
 #include "../../include/rbffd.h"
+#include "pool.cuh"
 
 namespace rbffd {
 
@@ -46,17 +47,6 @@ int device_sm_count();
 cudaError_t allow_smem(const void* fn, size_t bytes);
 
 // --------------------------------------------------- stream-ordered scratch
-// Stream-ordered allocations come from a memory pool of the library's own, one
-// per device.  The device's default pool gives everything back to the driver at
-// each synchronisation, so every call that ends with one - most here do - paid
-// 100 to 200 us to map its scratch again: set-up of a 10k-node problem (supports,
-// weights, plan, time step) 1.73 ms with it, 1.37 without.  The library's pool keeps at most
-// POOL_KEEP bytes that are not in use; what is above goes back at each
-// synchronisation, the rest when an allocation fails and when the library is unloaded.
-// Safe from any thread and stream (the driver orders reuse between streams).
-static constexpr unsigned long long POOL_KEEP = 128ull << 20;
-cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
-
 // RAII holder for pool memory; freed on the same stream.
 struct Scratch {
     void* p = nullptr;
