@@ -112,4 +112,22 @@ cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s) {
     return e;
 }
 
+void pool_free(void* const* p, int n) {
+    int first = 0, cur = 0;
+    while (first < n && !p[first]) ++first;
+    if (first == n) return;
+    cudaPointerAttributes a;
+    const bool known = cudaGetDevice(&cur) == cudaSuccess &&
+                       cudaPointerGetAttributes(&a, p[first]) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    const bool other = known && a.device != cur;
+    if (other) cudaSetDevice(a.device);
+    cudaDeviceSynchronize();
+    for (int i = first; i < n; ++i)
+        if (p[i]) cudaFreeAsync(p[i], cudaStreamPerThread);
+    // the pool gives back what it need not keep at a synchronisation, and not before
+    cudaStreamSynchronize(cudaStreamPerThread);
+    if (other) cudaSetDevice(cur);
+}
+
 }  // namespace rbffd

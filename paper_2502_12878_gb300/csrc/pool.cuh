@@ -17,4 +17,9 @@ namespace rbffd {
 static constexpr unsigned long long POOL_KEEP = 128ull << 20;
 cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
 
+// Frees up to n arrays of one device (null ones are skipped), whichever device is
+// current, when all work on theirs is done, as cudaFree would; what the pool then
+// holds above POOL_KEEP goes back before it returns.
+void pool_free(void* const* p, int n);
+
 }  // namespace rbffd

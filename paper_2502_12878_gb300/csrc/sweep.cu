@@ -828,12 +828,8 @@ static void drop_graphs(rbffd_plan* p) {
 
 static void free_plan(rbffd_plan* p) {
     if (!p) return;
-    if (p->slab) {
-        // nothing on the device uses it any more (cudaFree would wait, too)
-        cudaDeviceSynchronize();
-        cudaFreeAsync(p->slab, cudaStreamPerThread);
-        if (p->lk_slab) cudaFreeAsync(p->lk_slab, cudaStreamPerThread);
-    }
+    void* const slabs[] = {p->slab, p->lk_slab};
+    pool_free(slabs, 2);
     void* bufs[] = {p->nslot, p->ncol, p->nw, p->ng, p->ng0, p->uN, p->fl_idx[0], p->fl_idx[1],
                     p->fl_off[0], p->fl_off[1], p->fl_slot[0], p->fl_slot[1]};
     for (void* b : bufs)

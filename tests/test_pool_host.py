@@ -155,3 +155,31 @@ def test_contexts_and_pools(tmp_path):
         "full once: pool3 sync0 trim3 pool3 -> 0, device 0, context 2",
         "full: pool3 sync0 trim3 pool3 -> 2, device 0, context 2",
     ]
+
+
+FREES = r"""
+int main() {
+    void* a[3] = {0, (void*)(size_t)40, (void*)(size_t)50};       // of device 0
+    void* b[2] = {(void*)(size_t)1040, 0};                        // of device 1
+    cudaSetDevice(0);
+    trace.clear();
+    rbffd::pool_free(a, 3);
+    printf("%s| device %d\n", trace.c_str(), dev);
+    trace.clear();
+    rbffd::pool_free(b, 2);
+    printf("%s| device %d\n", trace.c_str(), dev);
+    trace.clear();
+    rbffd::pool_free(b + 1, 1);
+    printf("%s| device %d\n", trace.c_str(), dev);
+    return 0;
+}
+"""
+
+
+def test_frees_wait_for_the_arrays_own_device(tmp_path):
+    """... and give the memory back at once; the current device stays."""
+    assert _run(tmp_path, DRIVER.split("int main()")[0] + FREES) == [
+        "devsync0 free40 free50 sync0 | device 0",
+        "set1 devsync1 free1040 sync1 set0 | device 0",
+        "| device 0",
+    ]
