@@ -635,12 +635,13 @@ static int knn_impl(const double* xyz, int64_t N, int d, const uint8_t* cand,
     for (int a = 0; a < d; ++a) F.Rmax += (float)g.G[a];
     const double eps =
         F.eps_r * (double)F.R0 * F.R0 + (double)F.eps_0 * F.R0 + (double)F.eps_0 * F.eps_0;
-    const bool fast = 4.0 * eps < (double)F.R0 * F.R0 / KF_BINS;
+    bool fast = 4.0 * eps < (double)F.R0 * F.R0 / KF_BINS;
 
     Carve cv;
     const size_t o_start = cv.take(sizeof(int32_t) * (size_t)(ncell + 1));
     const size_t o_ids = cv.take(sizeof(int32_t) * (size_t)N);
     const size_t o_flags = cv.take(2 * sizeof(int));   // err, centres left to knn_kernel
+    const size_t slow_bytes = cv.used;
     const size_t o_count = fast ? cv.take(sizeof(int32_t) * (size_t)(ncell + 1)) : 0;
     const size_t o_tmp = fast ? cv.take(sizeof(int64_t) * (size_t)scan_tmp_elems(ncell)) : 0;
     const size_t o_key = fast ? cv.take(sizeof(int32_t) * (size_t)N) : 0;
@@ -649,7 +650,13 @@ static int knn_impl(const double* xyz, int64_t N, int d, const uint8_t* cand,
     const size_t o_sorted = fast ? cv.take(sizeof(float4) * (size_t)N) : 0;
     const size_t o_left = fast ? cv.take(sizeof(int32_t) * (size_t)nc) : 0;
     Scratch mem;
-    RBFFD_CHECK_CUDA(mem.alloc(cv.used, s));
+    cudaError_t e = mem.alloc(cv.used, s);
+    if (e == cudaErrorMemoryAllocation && fast) {   // knn_kernel needs a seventh of it
+        cudaGetLastError();
+        fast = false;
+        e = mem.alloc(slow_bytes, s);
+    }
+    RBFFD_CHECK_CUDA(e);
     char* base = mem.as<char>();
     int32_t* start = reinterpret_cast<int32_t*>(base + o_start);
     int32_t* ids = reinterpret_cast<int32_t*>(base + o_ids);

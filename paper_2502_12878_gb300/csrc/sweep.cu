@@ -1141,7 +1141,7 @@ link_lists(const int32_t* __restrict__ col, int64_t NI, int64_t N, int64_t nsl, 
 }
 
 // the lists, once per plan; lk_ok stays false where they, or the planes beside
-// them, do not fit
+// them, do not fit, or where there is no memory for them
 static int build_link(rbffd_plan* p, cudaStream_t s) {
     if (p->lk_built) return RBFFD_OK;
     p->lk_built = true;
@@ -1158,14 +1158,23 @@ static int build_link(rbffd_plan* p, cudaStream_t s) {
     if (N > LINK_MAX_N || link_smem(nsl, n, MODE_INNER32, G, 0) + 1024u > (unsigned)optin)
         return RBFFD_OK;
     const size_t map = 2 * sizeof(uint32_t) * (size_t)((N + 31) / 32);
-    RBFFD_CHECK_CUDA(allow_smem((const void*)link_lists, map));
+    if (allow_smem((const void*)link_lists, map) != cudaSuccess) {
+        cudaGetLastError();
+        return RBFFD_OK;
+    }
     const int64_t ent = nsl * n * SLICE;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t b_x = sizeof(unsigned long long) *
                        ((size_t)LINK_RING * 2 * NI + (size_t)LINK_RING * 2 * G + LINK_RING);
     const size_t o_off = up(b_x), o_slot = o_off + up(2 * sizeof(int32_t) * G),
                  o_idx = o_slot + up(sizeof(int32_t) * (size_t)G * LINK_CAP);
-    RBFFD_CHECK_CUDA(pool_alloc(&p->lk_slab, o_idx + sizeof(uint16_t) * ent, s));
+    const cudaError_t e = pool_alloc(&p->lk_slab, o_idx + sizeof(uint16_t) * ent, s);
+    if (e == cudaErrorMemoryAllocation) {   // the other launches need none of it
+        cudaGetLastError();
+        p->lk_slab = nullptr;
+        return RBFFD_OK;
+    }
+    RBFFD_CHECK_CUDA(e);
     char* base = (char*)p->lk_slab;
     p->lk_x = (unsigned long long*)base;
     p->lk_bytes = b_x;
