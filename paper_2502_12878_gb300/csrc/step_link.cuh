@@ -312,11 +312,10 @@ __global__ void __launch_bounds__(TH, 1) link_kernel(StepArgs A, StepCtrl* c) {
     if (!mbar_wait(mbar, 0, spin)) S.fail = 1;
     __syncthreads();
     if (S.fail) {
-        // give the copies a second bounded wait before the block leaves
         __syncthreads();
         if (threadIdx.x == 0) {
             atomicExch(&c->done, DONE_TIMEOUT);
-            mbar_wait(mbar, 0, spin);
+            mbar_drain(mbar, 0, spin);
         }
         __syncthreads();
         return;

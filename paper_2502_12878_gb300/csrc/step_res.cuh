@@ -75,6 +75,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
     }
 }
 
+// The wait of a block that gives up for its own copies in flight: they write its
+// shared memory, so it may not leave before they have landed, however short the
+// limit that ran out was (rbffd_plan_set_wait takes any; the planes' copies alone
+// take tens of microseconds).
+__device__ __forceinline__ void mbar_drain(uint32_t mbar, uint32_t parity, long long spin) {
+    constexpr long long least = SPIN_LIMIT_CYCLES;
+    mbar_wait(mbar, parity, spin > least ? spin : least);
+}
+
 // the iterate at slot c: from the block's halo window [lo, lo + W) in shared
 // memory, else a load through L1 (other blocks rewrite the iterate between steps,
 // each step behind an acquire)
@@ -359,10 +368,9 @@ __global__ void __launch_bounds__(TH, 1) resident_kernel(StepArgs A, StepCtrl* c
     if (!mbar_wait(mbar, 0, s_spin)) s_fail = 1;
     __syncthreads();
     if (s_fail) {
-        // give the copies a second bounded wait before the block leaves
         if (threadIdx.x == 0) {
             atomicExch(&c->done, DONE_TIMEOUT);
-            mbar_wait(mbar, 0, s_spin);
+            mbar_drain(mbar, 0, s_spin);
         }
         __syncthreads();
         return;
@@ -503,7 +511,7 @@ __global__ void __launch_bounds__(TH, 1) resident_kernel(StepArgs A, StepCtrl* c
         if (s_fail) {
             if (threadIdx.x == 0) {
                 atomicExch(&c->done, DONE_TIMEOUT);
-                mbar_wait(mbar, phase, spin);
+                mbar_drain(mbar, phase, spin);
             }
             __syncthreads();
             return;

@@ -136,6 +136,33 @@ def test_nonfinite_and_diverging_runs_end(rb, orc):
     assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("flag", ["RBFFD_LAUNCH_RESIDENT", "RBFFD_LAUNCH_FAR"])
+def test_limits_shorter_than_the_copies(rb, orc, flag):
+    """A wait limit below what the planes' copies into shared memory take: a block that gives up
+    still waits for them before it leaves.  Each solve ends with its result or as timed out."""
+    p = build(orc, 2, 120, 4, seed=11)
+    dt = 0.5 * 2.0 / np.abs(p.w).sum(1).max()
+    f, u0 = T(p.f), T(p.u0)
+    plan = rb.Plan(T(p.xyz), T(p.is_bnd), T(p.interior), T(p.idx), T(p.w), getattr(rb, flag), 3)
+    want = u0.clone()
+    plan.solve_explicit(f, want, dt, 50)
+    out = 0
+    for ms in (1e-5, 1e-4, 1e-3, 3e-3, 1e-2) * 6:
+        plan.set_wait(ms)
+        u = u0.clone()
+        try:
+            plan.solve_explicit(f, u, dt, 50)
+            assert torch.equal(u, want)
+        except rb.RbffdError as e:
+            assert e.code == rb.RBFFD_ERR_TIMEOUT
+            out += 1
+    assert out > 0
+    plan.set_wait()
+    u = u0.clone()
+    plan.solve_explicit(f, u, dt, 50)
+    assert torch.equal(u, want)
+
+
 def test_plans_of_different_sizes_share_kernels(rb, orc):
     """A launch's dynamic shared memory is limited by an attribute of the kernel: a smaller
     plan tuned later must not lower it below what a larger plan of the same kernel needs."""
