@@ -548,16 +548,34 @@ __device__ __forceinline__ void weights_one(const WeightArgs& A, int64_t r, doub
 // which share its FP64 pipe, and three on the others - so equal shares fixed in
 // advance leave three pipes idle while the fourth finishes: 1M stencils, s = 45
 // 94.8 -> 89.9 ms; s = 46 (twelve teams: three on each) 99.7 -> 97.9; s = 18
-// 12.3 -> 12.0.  Every team's first stencil is fixed - were it a ticket too, the
-// teams that start first would hold two while others get none (841 stencils of
-// s = 45 on 1976 teams 264 -> 418 us) - and consecutive ones go to different
-// blocks, so that few stencils spread over all SMs.  take_ticket draws
-// the next one after those (the team's first thread) and is called a stencil
-// ahead, which hides the atomic's latency; share_ticket tells the team.
-__device__ __forceinline__ long long take_ticket(unsigned long long* tickets, int tid,
+// 12.3 -> 11.8.  Every team's first stencil is fixed (first_stencil).  take_ticket
+// draws the next one after those (the team's first thread) and share_ticket tells
+// the team.  A ticket is drawn when the stencil before it is done: drawn a stencil
+// ahead, the last ones are held by busy teams, all of them on the SMs that started
+// first, while other SMs have none (s = 46, 2025 stencils 430 us against 383; s = 30,
+// 4913 354 against 307).  In long builds that matters less than the latency of the
+// atomic (s = 45, 489k stencils: 44.1 ms ahead, 44.3 not), so one-warp teams draw
+// ahead (AHEAD) from WEIGHT_AHEAD stencils a team on.  Five-warp teams, two or
+// three on an SM, are equally fast; below WEIGHT_SHARES stencils a team their shares
+// are fixed, r, r + teams, ..., which spreads the last ones over the SMs where a
+// ticket goes to whole SMs in turn (s = 84, 1089 stencils 867 us against 830; in
+// longer builds tickets gain 1 %).
+static constexpr int WEIGHT_AHEAD = 16, WEIGHT_SHARES = 8;
+
+template <int TS>
+__device__ __forceinline__ long long take_ticket(unsigned long long* tickets, int tid, int64_t r,
                                                  int64_t teams, int64_t total) {
+    if (TS > 32 && total <= WEIGHT_SHARES * teams) return (long long)(r + teams);
     if (teams >= total) return (long long)total;   // (the counter is not used, nor set)
     return tid == 0 ? (long long)teams + (long long)atomicAdd(tickets, 1ull) : 0ll;
+}
+// The first stencils: as many as a warp holds teams to each warp (a warp costs the
+// FP64 pipe the same with half its lanes idle), and consecutive warps' to different
+// blocks, so that few stencils spread over all SMs.
+template <int TS>
+__device__ __forceinline__ int64_t first_stencil(int team) {
+    constexpr int W = TS < 32 ? 32 / TS : 1;
+    return (blockIdx.x + (int64_t)(team / W) * gridDim.x) * W + team % W;
 }
 template <int TS>
 __device__ __forceinline__ int64_t share_ticket(long long v, int tid, int team,
@@ -572,7 +590,7 @@ __device__ __forceinline__ int64_t share_ticket(long long v, int tid, int team,
     }
 }
 
-template <int TS, bool PW>
+template <int TS, bool PW, bool AHEAD>
 __global__ void __launch_bounds__(weight_max_threads(TS))
     weights_kernel(WeightArgs A, unsigned long long* tickets) {
     extern __shared__ double wsm[];
@@ -587,10 +605,12 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
     double* xi = G + (size_t)A.s * A.pitch;
     __shared__ long long s_next[16];
     const int64_t teams = (int64_t)gridDim.x * (blockDim.x / TS);
-    int64_t r = blockIdx.x + (int64_t)team * gridDim.x;
+    int64_t r = first_stencil<TS>(team);
     while (r < A.nc) {
-        const long long ticket = take_ticket(tickets, tid, teams, A.nc);
+        long long ticket = 0;
+        if constexpr (AHEAD) ticket = take_ticket<TS>(tickets, tid, r, teams, A.nc);
         weights_one<TS, PW>(A, r, G, xi, tid, team, redv, redk, redi, bcast, spiv);
+        if constexpr (!AHEAD) ticket = take_ticket<TS>(tickets, tid, r, teams, A.nc);
         r = share_ticket<TS>(ticket, tid, team, s_next);
     }
 }
@@ -598,7 +618,7 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
 // many calls in one launch: stencil number g of the concatenation belongs to
 // the call dI with off[dI] <= g < off[dI + 1]; a team's shared memory holds
 // the largest system of the launch (team_doubles)
-template <int TS, bool PW>
+template <int TS, bool PW, bool AHEAD>
 __global__ void __launch_bounds__(weight_max_threads(TS))
     weights_multi_kernel(const WeightArgs* __restrict__ calls, const int64_t* __restrict__ off,
                          int ncalls, unsigned long long* tickets, int64_t team_doubles) {
@@ -614,9 +634,10 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
     __shared__ long long s_next[16];
     const int64_t total = off[ncalls];
     const int64_t teams = (int64_t)gridDim.x * (blockDim.x / TS);
-    int64_t g = blockIdx.x + (int64_t)team * gridDim.x;
+    int64_t g = first_stencil<TS>(team);
     while (g < total) {
-        const long long ticket = take_ticket(tickets, tid, teams, total);
+        long long ticket = 0;
+        if constexpr (AHEAD) ticket = take_ticket<TS>(tickets, tid, g, teams, total);
         int lo = 0, hi = ncalls - 1;   // last call with off <= g
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -626,6 +647,7 @@ __global__ void __launch_bounds__(weight_max_threads(TS))
         const WeightArgs& A = calls[lo];
         double* xi = G + (size_t)A.s * A.pitch;
         weights_one<TS, PW>(A, g - off[lo], G, xi, tid, team, redv, redk, redi, bcast, spiv);
+        if constexpr (!AHEAD) ticket = take_ticket<TS>(tickets, tid, g, teams, total);
         g = share_ticket<TS>(ticket, tid, team, s_next);
     }
 }
@@ -673,15 +695,15 @@ typedef void (*WeightMultiKernel)(const WeightArgs*, const int64_t*, int, unsign
                                   int64_t);
 
 // the five-warp team has a pivot warp
-static WeightKernel weight_kernel_for(int ts) {
-    if (ts == 16) return weights_kernel<16, false>;
-    if (ts == 32) return weights_kernel<32, false>;
-    return weights_kernel<160, true>;
+static WeightKernel weight_kernel_for(int ts, bool ahead) {
+    if (ts == 16) return weights_kernel<16, false, false>;
+    if (ts == 32) return ahead ? weights_kernel<32, false, true> : weights_kernel<32, false, false>;
+    return weights_kernel<160, true, false>;
 }
-static WeightMultiKernel weight_multi_kernel_for(int ts) {
-    if (ts == 16) return weights_multi_kernel<16, false>;
-    if (ts == 32) return weights_multi_kernel<32, false>;
-    return weights_multi_kernel<160, true>;
+static WeightMultiKernel weight_multi_kernel_for(int ts, bool ahead) {
+    if (ts == 16) return weights_multi_kernel<16, false, false>;
+    if (ts == 32) return ahead ? weights_multi_kernel<32, false, true> : weights_multi_kernel<32, false, false>;
+    return weights_multi_kernel<160, true, false>;
 }
 
 struct WeightShape {
@@ -721,6 +743,15 @@ static cudaError_t pick_weight_shape(K kern, int ts, size_t per_team, WeightShap
     b.smem = per_team * b.tpb;
     *out = b;
     return cudaSuccess;
+}
+
+// blocks for `total` stencils: as many for every SM as its share of them needs
+// when their warps are full
+static int64_t weight_grid(const WeightShape& ws, int sms, int64_t total) {
+    const int w = ws.ts < 32 ? 32 / ws.ts : 1;        // stencils of a warp
+    const int64_t warps = (total + w - 1) / w;
+    const int64_t per_sm = ((warps + sms - 1) / sms + ws.tpb / w - 1) / (ws.tpb / w);
+    return std::min<int64_t>(warps, sms * std::min<int64_t>(per_sm, ws.per_sm));
 }
 
 // monomial exponents of degree <= m in graded order: degree ascending, then
@@ -783,10 +814,13 @@ static int weights_impl(const double* xyz, int64_t N, int d, const int32_t* idx,
     const int sms = device_sm_count();
     WeightShape ws;
     const int ts = weight_team_size(A.s);
-    WeightKernel kern = weight_kernel_for(ts);
+    WeightKernel kern = weight_kernel_for(ts, false);
     RBFFD_CHECK_CUDA(pick_weight_shape(kern, ts, per_team, &ws));
-    // (a block a stencil up to what is resident: the first stencils go to different blocks)
-    const int64_t grid = std::min<int64_t>(nc, (int64_t)sms * ws.per_sm);
+    const int64_t grid = weight_grid(ws, sms, nc);
+    if (nc >= WEIGHT_AHEAD * grid * ws.tpb) {
+        kern = weight_kernel_for(ts, true);
+        RBFFD_CHECK_CUDA(allow_smem((const void*)kern, ws.smem));
+    }
     Scratch cnt;   // singular stencils, the first of them, the teams' tickets
     RBFFD_CHECK_CUDA(cnt.alloc(3 * sizeof(unsigned long long), s));
     if (grid * ws.tpb < nc)   // (else no team takes a ticket)
@@ -892,9 +926,13 @@ extern "C" int rbffd_weights_batch(int ncalls, const double* const* xyz, const i
         for (const WeightArgs& A : sel) max_s = std::max(max_s, A.s);
         WeightShape ws;
         const int ts = weight_team_size(max_s);
-        WeightMultiKernel kern = weight_multi_kernel_for(ts);
+        WeightMultiKernel kern = weight_multi_kernel_for(ts, false);
         RBFFD_CHECK_CUDA(pick_weight_shape(kern, ts, per_team, &ws));
-        const int64_t grid = std::min<int64_t>(off.back(), (int64_t)sms * ws.per_sm);
+        const int64_t grid = weight_grid(ws, sms, off.back());
+        if (off.back() >= WEIGHT_AHEAD * grid * ws.tpb) {
+            kern = weight_multi_kernel_for(ts, true);
+            RBFFD_CHECK_CUDA(allow_smem((const void*)kern, ws.smem));
+        }
         Scratch tickets;
         RBFFD_CHECK_CUDA(tickets.alloc(sizeof(unsigned long long), s));
         RBFFD_CHECK_CUDA(cudaMemsetAsync(tickets.p, 0, sizeof(unsigned long long), s));

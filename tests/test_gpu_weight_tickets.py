@@ -26,3 +26,18 @@ def test_counts(rb, d, Kg, m, n):
     for k in (1, 2, 7, 151, 152, 153, 303, 841, 1975, 1976, 1977, 2432, 3953, idx.shape[0] - 1):
         if k < idx.shape[0]:
             assert torch.equal(rb.rbffd_weights(xyz, idx[-k:].contiguous(), m)[0], w[-k:])
+
+
+@pytest.mark.parametrize("d,Kg,m,n", [(2, 200, 4, 30), (2, 200, 4, 31), (2, 140, 2, 13),
+                                      (2, 70, 6, 57), (3, 16, 4, 71)])
+def test_long_and_short_builds(rb, d, Kg, m, n):
+    """Builds on either side of the rounds of stencils at which teams begin to draw tickets ahead
+    or to draw them at all, one call and several calls in one launch."""
+    xyz, bnd = rb.rbffd_nodes(d, 0, Kg, 0.3, 2)
+    idx = rb.rbffd_knn(xyz, rb.rbffd_interior(bnd), n)
+    w, _ = rb.rbffd_weights(xyz, idx, m)
+    cuts = [0, 1, 33, 900, 2001, idx.shape[0]]
+    parts = [idx[a:b].contiguous() for a, b in zip(cuts, cuts[1:])]
+    assert torch.equal(torch.cat([rb.rbffd_weights(xyz, p, m)[0] for p in parts]), w)
+    both = rb.rbffd_weights_batch([xyz] * len(parts), parts, [m] * len(parts))
+    assert torch.equal(torch.cat([x for x, _ in both]), w)
