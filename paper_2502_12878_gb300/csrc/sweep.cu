@@ -1770,16 +1770,22 @@ extern "C" int rbffd_apply(const double* w, const int32_t* idx, int64_t nc, int 
     if (nc == 0) return RBFFD_OK;
     RBFFD_ARG(w && idx && u && Lu, "rbffd_apply: NULL argument");
     int sms = device_sm_count();
-    // whole-row tiles where the 16-byte copies may start at every tile and a
-    // tile fits a block's shared memory (n <= 586); else a thread per row
+    // whole-row tiles where the 16-byte copies may start at every tile, a tile fits a
+    // block's shared memory (n <= 586), and at least three do (n <= 196) or the call has
+    // no more than two and a half tiles for each that is resident: else a thread per
+    // row, which keeps more loads in flight.  Thread per row against tiles, 90k rows: n = 148
+    // 74 against 67 us, 200 114 and 136, 400 284 and 481, 580 286 and 611; 400k rows of
+    // 196 442 and 341; 10k rows of 400 (2.1 tiles each) 96 and 73, 20k (4.1) 100 and
+    // 120.  (Three tiles, even n, 30k to 150k rows: between 0.85 and 1.3 of the thread
+    // per row's speed, as the tiles happen to divide.)
     const size_t smem = (size_t)APPLY_WARPS * SLICE * n * 12;
-    if (smem <= 220 * 1024 &&
+    const int64_t ntiles = (nc + SLICE - 1) / SLICE;
+    const int64_t per_sm = std::min<int64_t>(32, (227 * 1024) / (int64_t)(smem + 1024));
+    if (smem <= 220 * 1024 && (per_sm >= 3 || 2 * ntiles <= 5 * sms * per_sm) &&
         (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(idx)) % 16 == 0) {
         const void* fn = n % 2 ? (const void*)apply_tiles<1> : (const void*)apply_tiles<2>;
         if (smem > 48 * 1024)
             RBFFD_CHECK_CUDA(allow_smem(fn, smem));
-        const int64_t ntiles = (nc + SLICE - 1) / SLICE;
-        const int64_t per_sm = std::min<int64_t>(32, (227 * 1024) / (int64_t)(smem + 1024));
         const int64_t grid =
             std::min<int64_t>((ntiles + APPLY_WARPS - 1) / APPLY_WARPS, (int64_t)sms * per_sm);
         void* args[] = {(void*)&w, (void*)&idx, (void*)&nc, (void*)&n, (void*)&u, (void*)&Lu};

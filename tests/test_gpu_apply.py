@@ -35,3 +35,19 @@ def test_apply_tiles(rb, orc, rows, n, skip):
     ref = orc.apply(np.ascontiguousarray(w[skip:]), np.ascontiguousarray(idx[skip:]), u)
     scale = np.maximum(np.abs(ref), (np.abs(w[skip:]) * np.abs(u[idx[skip:]])).sum(1))
     assert np.all(np.abs(got - ref) <= 1e-12 * scale)
+
+
+@pytest.mark.parametrize("n", [196, 197, 199, 200, 301, 400])
+def test_long_rows_by_either_kernel(rb, n):
+    """Rows of a length of which few tiles fit an SM go to one kernel or the other by their
+    number: each row's chain, and so its bits, are the same."""
+    g = torch.Generator("cuda").manual_seed(n)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    fit = (227 * 1024) // (32 * n * 12 + 1024)
+    for rows in (16 * 5 * sms * fit // 32 * 32, 16 * 5 * sms * fit // 32 * 32 + 1, 40000):
+        w = torch.randn((rows, n), generator=g, device="cuda", dtype=torch.float64)
+        idx = torch.randint(0, rows, (rows, n), generator=g, device="cuda", dtype=torch.int32)
+        u = torch.randn(rows, generator=g, device="cuda", dtype=torch.float64)
+        cut = rows // 64 * 32
+        parts = [rb.rbffd_apply(w[a:b], idx[a:b], u) for a, b in ((0, cut), (cut, rows))]
+        assert torch.equal(rb.rbffd_apply(w, idx, u), torch.cat(parts))
