@@ -6,11 +6,13 @@
  *
  * Conventions, for every entry point:
  *  - Pointers are DEVICE pointers unless the name starts with h_ (host).
- *    All arrays are caller-owned; the library never frees them.  The only
+ *    All arrays are caller-owned; the library never frees them.  The
  *    memory the library owns is inside an rbffd_plan (freed by
- *    rbffd_plan_destroy) and short-lived scratch taken from the stream-ordered
- *    allocator (cudaMallocAsync on the given stream) and returned before the
- *    call returns.
+ *    rbffd_plan_destroy) and short-lived scratch, stream-ordered on the given
+ *    stream and returned before the call returns.  Both come from a memory pool
+ *    of the library's own, one per device, which keeps up to 128 MB that are
+ *    not in use (in a context that is not the device's primary one: from the
+ *    device's default pool).
  *  - Coordinates are structure-of-arrays FP64: xyz[a * N + i] is coordinate a
  *    (a < d) of node i.  Node indices are int32.
  *  - `stream` is a cudaStream_t (NULL = legacy default stream).  Work is
@@ -131,10 +133,12 @@ RBFFD_API int rbffd_nodes(int d, int shape, int Kg, double jitter_frac, uint64_t
  *   xyz      [d][cap] FP64 device out; is_bnd [cap] device out (1 seeds,
  *            0 the rest); seeds first, then the walk's appends in order
  *   h_n_out  host: number of nodes; RBFFD_ERR_CAPACITY if it exceeds cap
- *   h_rounds host [2] (may be NULL): generations walked, and conflict-
- *            resolution passes over all generations
- * Synchronises `stream` (2D: once per 16 generations; 3D: a few times per
- * generation); scratch comes from cudaMallocAsync on `stream`.
+ *   h_rounds host [2] (may be NULL): generations walked, and the rounds of
+ *            conflict resolution (2D: the most looks a warp of the deciding
+ *            block took) summed over all generations
+ * Synchronises `stream` (2D: once or twice; 3D: a few times per generation).
+ * The 2D walk is one cooperative launch: it starts when the whole GPU is free, and
+ * its waits between blocks end after about 2 s (RBFFD_ERR_TIMEOUT).
  */
 RBFFD_API int rbffd_nodes_pds(int d, int shape, int Kg, int K, double zeta, uint64_t seed,
                               double* xyz, uint8_t* is_bnd, int64_t cap, int64_t* h_n_out,
@@ -161,8 +165,8 @@ RBFFD_API int rbffd_interior(const uint8_t* is_bnd, int64_t N, int32_t* interior
  * Row r lists its n nodes by increasing key (d2, j), where
  * d2 = fl(fl(dx0*dx0) + fl(dx1*dx1) [+ fl(dx2*dx2)]), dx = fl(x_j - x_c), so
  * equal distances are ordered by node index and the centre comes first.
- * Uses a uniform cell grid (counting sort) and ring search; scratch comes
- * from cudaMallocAsync on `stream`.
+ * Uses a uniform cell grid (counting sort); candidates are ordered by FP32
+ * distances with an error bound, and by the FP64 keys where it leaves them open.
  */
 RBFFD_API int rbffd_knn(const double* xyz, int64_t N, int d, const int32_t* centres, int64_t nc, int n,
               int32_t* idx, void* stream);
@@ -326,8 +330,9 @@ RBFFD_API int rbffd_fp64_fma_rate(int64_t iters, double* h_fma_per_s, double* h_
  * RBFFD_ERR_CAPACITY from its first solve.  Unless a reach is fixed by
  * rbffd_plan_set_resident_halo, _RESIDENT and _AUTO plans that fit run it linked:
  * blocks pass each other the rows that they read, tagged with their step, so that
- * a step waits for its neighbours' rows instead of a barrier of all blocks (16 x 8
- * bytes a row of device memory more).  A Morton plan created with a
+ * a step waits for its neighbours' rows instead of a barrier of all blocks (128 + 2 n
+ * bytes a row and 16 KB a block of device memory more; without that memory the plan
+ * takes another launch).  A Morton plan created with a
  * flag that allows the resident or split launch, whose share per SM is at
  * least two slices and fits one of them, orders each share's rows with the
  * rows whose supports lie inside the share first, each group in Morton
@@ -366,8 +371,10 @@ RBFFD_API int rbffd_plan_set_neumann(rbffd_plan* plan, int64_t NN, const int32_t
  * device's maximum clock, and the solve then returns RBFFD_ERR_TIMEOUT.
  * held_arrivals (0..1024, normally 0) is a failure injection for testing that
  * path: the barrier waits for that many arrivals beyond the grid's (linked: the
- * stop decisions are withheld), which never come, so every block gives up after the timeout and returns.  Takes
- * effect from the next solve; graph-mode steps have no waits.
+ * stop decisions are withheld), which never come, so every block gives up after
+ * the timeout and returns.  Takes effect from the next solve; graph-mode steps
+ * have no waits.  rbffd_stable_dt's waits have the same limit, and it goes on
+ * without them where they run out.
  */
 RBFFD_API int rbffd_plan_set_wait(rbffd_plan* plan, double timeout_ms, int held_arrivals);
 /*
@@ -553,7 +560,7 @@ RBFFD_API int rbffd_stable_dt(rbffd_plan* plan, const double* v0, int iters, dou
  * rows, same bits, fewer bytes), else each entry's position in the slice,
  * through which its int32 row is read.  Owned by
  * the plan (freed by rbffd_plan_destroy); a second call does nothing.
- * Synchronises `stream`; scratch comes from cudaMallocAsync on `stream`.
+ * Synchronises `stream`.
  */
 RBFFD_API int rbffd_transpose(rbffd_plan* plan, void* stream);
 

@@ -493,7 +493,9 @@ __global__ void adj_outputs(const double* S, const double* lam, const int32_t* r
 // interior rows updated, boundary slots copied.  The forward sweep's row sums
 // (step.cuh: 16-bit neighbour codes, fixed lengths, loads in phases, 64
 // registers), so the replayed iterates are the forward's bit for bit, and a
-// programmatic dependent launch.  Bound like the sweep by the FP64 pipe and
+// programmatic dependent launch.  (At n = 40 and 48 64 registers spill 88 and 132
+// bytes a thread; sizes without a kernel of their own keep predicated phases of
+// eight over the int32 indices.)  Bound like the sweep by the FP64 pipe and
 // latency; with wgrad_group's sums of whole groups a step of rbffd_adjoint_w (K = 64,
 // spacing 8) went at 9.8k rows, n = 12 from 20.8 to 10.8 us, at 89k, n = 30 from 40.8
 // to 31.7, at 1M from 267 to 209 (phases of eight over the 16-bit codes at any

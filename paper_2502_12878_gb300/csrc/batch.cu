@@ -399,7 +399,8 @@ __device__ bool run_domain(const TeamDesc T, const DomDesc* __restrict__ desc,
 // plane's latency and the prefetch's L2 requests only compete.  20 domains of
 // 5k..100k nodes, n = 12, 30 and 56, 200 steps, kernel time: 1024-thread
 // blocks 11.66 -> 9.88 ms, of which the weak loads 0.26, leaving out the
-// prefetch 0.64, phases of 20 instead of 8 0.37 (16: 0.23; 24, 28 and 56 give
+// prefetch (n = 30 and 56; the kernel for run-time sizes keeps it, whatever n: not
+// measured without) 0.64, phases of 20 instead of 8 0.37 (16: 0.23; 24, 28 and 56 give
 // some or all of it back) and brow's phases 0.47; two blocks of 512 10.98 ->
 // 9.64.  With more registers and so fewer warps the prefetch and .cg stay: L1
 // took 512-thread blocks with 128 registers from 12.5 to 13.3 ms, without the

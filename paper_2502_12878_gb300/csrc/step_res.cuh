@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(TH, 1) resident_kernel(StepArgs A, StepCtrl* c
     // the halo window: the block's rows and A.halo slots on either side, its
     // start rounded down and its length down to 16-byte multiples (a TMA bulk
     // copy's rule), within [0, N)
-    // (A.halo < 0: no window, every gather through L2)
+    // (A.halo < 0: no window, every gather from memory)
     const int64_t lo64 = max((int64_t)0, s0 * SLICE - A.halo) & ~(int64_t)3;
     const int64_t hi64 = min(A.N, s1 * SLICE + A.halo);
     const uint32_t W =
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(TH, 1) resident_kernel(StepArgs A, StepCtrl* c
                 const int32_t row = r0i + ord[i] * SLICE + lane;
                 if (row < NI32) unext[row] = o_next[row - r0i];
             }
-        // far values: plain loads through L2 (acquired at the barrier like the
+        // far values: plain loads (acquired at the barrier like the
         // window's source), stored behind the window - other addresses than
         // the bulk copy's, ordered for the readers by the barrier below
         if constexpr (FAR)

@@ -8,7 +8,7 @@
 // the previous step; their results go to the iterate once that barrier has
 // passed (a slower block may still be reading the buffer they overwrite).
 // Then all warps compute the remaining slices, gathering the other shares'
-// rows through L2.  The stencil planes are streamed as in the one-launch-
+// rows with loads that L1 may serve (the barrier's acquire drops what it held).  The stencil planes are streamed as in the one-launch-
 // per-step kernel, and each row's arithmetic is the same fused multiply-add
 // chain, so the results are the same bit for bit.
 #pragma once
@@ -24,7 +24,7 @@ __host__ __device__ __forceinline__ unsigned split_smem_bytes(int64_t nsl, int w
 
 // sum_j w_j u[col_j], the planes streamed (indices, weights, then the
 // gathers, CH at a time, as row_dot); the iterate from the own-row buffer o
-// (at c - r0) where the column is a row of the block, else through L2.  OWN:
+// (at c - r0) where the column is a row of the block, else from memory.  OWN:
 // every column is.
 template <int NN, bool OWN, bool I16, int CH, class T>
 __device__ __forceinline__ T row_dot_split(const T* __restrict__ w, const void* __restrict__ colp,
@@ -89,8 +89,11 @@ __device__ __forceinline__ T split_row(const StepArgs& A, int64_t sl, int32_t ro
     const int64_t base = sl * (int64_t)A.n * SLICE + lane;
     const int4 sb = A.col16 ? __ldg(A.sbase + sl) : make_int4(-1, -1, -1, -1);
     // loads in flight per thread: fewer for the generic size and in the FP64
-    // 1024-thread blocks (64 registers), so nothing spills (12 fit from n = 30
-    // on, 8 for the smaller sizes: by the compiler's register report)
+    // 1024-thread blocks (64 registers), so the compiled sizes do not spill (12 fit
+    // from n = 30 on, 8 for the smaller ones: by the compiler's register report).
+    // The generic size (NN = 0) still has its phases under j < n and spills their
+    // predicates (372 bytes in the FP64 kernel): 90k rows of n = 21 20 us a step
+    // where the other launches take 7 to 8
     constexpr int CH = NN == 0                                    ? 8
                        : !(MODE == MODE_SWEEP64 && TH >= 1024)    ? 16
                        : NN >= 30                                 ? 12
@@ -259,7 +262,7 @@ __global__ void __launch_bounds__(TH, 1) split_kernel(StepArgs A, StepCtrl* c) {
                 if (row < NI32) unext[row] = o_next[row - r0];
             }
         // the other slices, one at a time from the shared counter: the other
-        // shares' rows of u^k through L2
+        // shares' rows of u^k through L1 and L2
         for (;;) {
             int i = 0;
             if (lane == 0) i = atomicAdd(&s_next, 1);

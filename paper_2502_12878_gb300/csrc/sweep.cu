@@ -1265,9 +1265,10 @@ static int tune_shape(rbffd_plan* p, int mode, cudaStream_t s) {
     // the linked launch, wherever the resident one may be chosen (not when
     // rbffd_plan_set_resident_halo fixed a reach: that asks for its window).
     // Where no block reads more than LINK_ONLY slots of others it is taken
-    // without timing the other launches: measured from 1.5k to 89k rows, n = 12 to
-    // 70, 2D and 3D, Morton and random orders, the best of them took 1.13 to 2.5
-    // times as long; above (a random order of 3D supports: 2,500 slots) it may lose
+    // without timing the other launches: measured from 361 to 89k rows, n = 9 to
+    // 100, 2D and 3D, Morton and random orders, the best of them took 1.04 to 2.5
+    // times as long (one exception found: 89k rows of n = 17, without a kernel of their
+    // own, in FP64 6.9 us in the persistent launch against 7.1); above (a random order of 3D supports: 2,500 slots) it may lose
     // (5.8 us against 5.6).
     bool link_only = false;
     if (may_persist(p) && !only_split && !only_far &&
@@ -1959,7 +1960,12 @@ extern "C" int rbffd_plan_create(const double* xyz, const uint8_t* is_bnd, int64
     p->nslices = (NI + SLICE - 1) / SLICE;
     p->grid_steps = 2;
     const size_t ell = (size_t)p->nslices * n * SLICE;
-    // every array of the plan in one allocation, each on a 256-byte boundary
+    // every array of the plan in one allocation, each on a 256-byte boundary.  (Where
+    // the arrays lie decides some per cent of a sweep whose planes about fill L2, from
+    // one plan to the next: medians over placements, an allocation each against this,
+    // FP32 steps of 490k rows 10.1 against 10.5 us at n = 20, 7.0 and 7.1 at 13, 6.35
+    // and 6.4 at 12, 160k rows of 56 8.5 and 8.4, 250k of 12 6.5 either way; making a plan
+    // of 250k rows 1.1 ms and freeing it 0.5 against 0.26 and 0.01.)
     const int sm_count = device_sm_count();
     const bool inner = inner_first_applies(p, flags), codes = !(flags & RBFFD_PACK_IDX32);
     cudaError_t e = cudaSuccess;
